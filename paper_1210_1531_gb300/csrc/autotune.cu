@@ -30,7 +30,7 @@ int autotune_impl(elses_system s, cudaStream_t st) {
         bool split = false;
         for (int a = 0; a < s->n; ++a) {
             const int k = (s->h_clsize[a] + 15) / 16;
-            if ((k & 1) && k < (int)s->tuned_half.size() && !s->tuned_half[k]) {
+            if ((k & 1) && k < (int)s->tuned_half.size() && !s->tuned_half[k] && !s->fx) {
                 s->tuned_half[k] = 1;
                 split = true;
             }
@@ -51,15 +51,17 @@ int autotune_impl(elses_system s, cudaStream_t st) {
         // with half-warps (capacity 16 ns) or with whole warps (capacity 16 (ns + 1))
         struct Form { int half, na, maxb; };
         std::vector<Form> forms;
-        if (half_ok && (ns & 1)) forms = {{1, 16 * ns, 0}, {0, 16 * (ns + 1), 0}};
+        if (half_ok && (ns & 1) && L.fx < 0) forms = {{1, 16 * ns, 0}, {0, 16 * (ns + 1), 0}};
         else forms = {{L.half, L.na, 0}};
         int maxb_all = 0;
         for (auto& f : forms) {
-            f.maxb = s->p.krylov_block ? block_krylov_blocks_per_sm(f.na, kdeg)
+            f.maxb = L.fx >= 0         ? fx_blocks_per_sm(L.fx, f.na, s->max_nb, nm, s->p.reorth != 0, s->p.force_mode == 1)
+                     : s->p.krylov_block ? block_krylov_blocks_per_sm(f.na, kdeg)
                      : f.half          ? krylov_half_blocks_per_sm(f.na, kdeg)
                                        : krylov_blocks_per_sm_max(f.na, kdeg);
             maxb_all = std::max(maxb_all, f.maxb);
-            const size_t per_cta = s->p.krylov_block ? block_krylov_scratch_doubles(nm, f.na)
+            const size_t per_cta = L.fx >= 0         ? fx_scratch_doubles(L.fx, nm, f.na)
+                                   : s->p.krylov_block ? block_krylov_scratch_doubles(nm, f.na)
                                                      : (size_t)kWarpsPerAtom * 2 * nm * f.na * 4;
             if ((rc = s->kscratch.ensure((size_t)s->num_sms * f.maxb * per_cta)) < 0) break;
         }
@@ -79,7 +81,7 @@ int autotune_impl(elses_system s, cudaStream_t st) {
             ka.order = s->order.p + L.item_begin;
             ka.n_items = sample;
             ka.scratch = s->kscratch.p;
-            const int grid = std::min(sample, s->num_sms * b);
+            const int grid = std::min(L.fx >= 0 ? fx_items(L.fx, sample) : sample, s->num_sms * b);
             float ms = 0.f;
             for (int rep = 0; rep < 2; ++rep) {       // the first launch warms caches and clocks
                 if (s->p.schedule == 1) {
@@ -87,8 +89,7 @@ int autotune_impl(elses_system s, cudaStream_t st) {
                     if (cudaMemsetAsync(ka.queue, 0, sizeof(int), st) != cudaSuccess) { rc = fail(ELSES_ERR_CUDA, "memset"); break; }
                 }
                 cudaEventRecord(e0, st);
-                if (s->p.krylov_block) block_krylov_columns(ka, grid, st);
-                else krylov_columns(ka, grid, b, st);
+                launch_krylov(s, ka, L.fx, grid, b, st);
                 cudaEventRecord(e1, st);
                 s->stats.launches++;
             }
@@ -125,12 +126,11 @@ int autotune_impl(elses_system s, cudaStream_t st) {
             ka.n_items = L.item_count;
             ka.scratch = s->kscratch.p;
             ka.queue = s->counters.p + kQueue0;
-            const int grid = std::min(L.item_count, s->num_sms * best_b);
+            const int grid = std::min(L.fx >= 0 ? fx_items(L.fx, L.item_count) : L.item_count, s->num_sms * best_b);
             for (int rep = 0; rep < 2; ++rep) {
                 cudaMemsetAsync(ka.queue, 0, sizeof(int), st);
                 cudaEventRecord(e0, st);
-                if (s->p.krylov_block) block_krylov_columns(ka, grid, st);
-                else krylov_columns(ka, grid, best_b, st);
+                launch_krylov(s, ka, L.fx, grid, best_b, st);
                 cudaEventRecord(e1, st);
                 s->stats.launches++;
             }

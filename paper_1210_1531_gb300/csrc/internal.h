@@ -48,6 +48,21 @@ void cohp_spectrum(const double* pos, const double L[3], const SKDev& sk, const 
                    double* Csig, double* Cpi, cudaStream_t st);
 
 // ---------------------------------------------------------------- a3, a4 (krylov.cu)
+// Scales of the fixed-point form's coefficients (krylov_fixed.cu): a coefficient c is the integer
+// c 2^eH (eS for the overlap).
+struct FxScale {
+    int ok;                 // 0: the system's coefficients do not suit the fixed-point form
+    int eH, eS;
+    int2 Es, Ep, one;       // on-site energies of H and the on-site 1 of S
+};
+struct FxArgs {
+    const int4* rec;        // [nnzb][6] block records
+    const FxScale* scale;
+    double Es, Ep;          // on-site energies
+    int smem_bytes;         // dynamic shared memory of the launch
+    int split;              // 1: the CTAs take an atom's column groups as separate items
+};
+
 struct KrylovArgs {
     int n_atoms;
     const int* row_ptr;
@@ -112,6 +127,15 @@ struct AdjointArgs {
     const double* bstore;   // bases kept by the energy pass (KrylovArgs layout), or nullptr:
     size_t bstride, bvec;   // then the forward recursion is recomputed
 };
+// fixed-point form (krylov_fixed.cu): scales and block records of a Slater-Koster system (bounds:
+// six words), then the launch of a size class
+void fx_build(int n, int nnzb, const int* row_ptr, const int* col_idx, const double* skr, double Es, double Ep,
+              int max_row, unsigned long long* bounds, FxScale* scale, int2* rec, cudaStream_t st);
+int fx_form_for(int n, int sms);                       // for a system of n atoms
+int fx_items(int form, int count);                     // CTAs' work items of it
+int fx_blocks_per_sm(int form, int na, int max_row, int nu, bool overlap, bool store);   // 0: the class does not fit
+size_t fx_scratch_doubles(int form, int nu, int na);   // per resident CTA
+void fx_columns(const KrylovArgs& a, FxArgs x, int form, int grid, int ctas_per_sm, cudaStream_t st);
 size_t krylov_smem_bytes(int na_max, int deg_max);
 int krylov_blocks_per_sm(int na_max, int deg_max);       // resident CTAs at the 3-CTA register budget
 int krylov_blocks_per_sm_max(int na_max, int deg_max);   // with the 4-CTA form where shared memory allows

@@ -117,6 +117,7 @@ int prepare_columns(elses_system s) {
     // warps per SM as k_krylov at capacity 16 (c + 1), or as the autotuner chose; the others run
     // k_krylov. Otherwise slots of 32.
     const bool half_ok = s->p.k3_lanes != 32 && s->p.force_mode == 0 && !s->p.krylov_block;
+    const bool fx_ok = s->fx && !s->user_hs && !s->p.krylov_block;
     const int gslot = half_ok ? 16 : 32;
     std::vector<int> ord;
     ord.reserve(s->n);
@@ -131,7 +132,7 @@ int prepare_columns(elses_system s) {
     };
     for (int b = 0; b < s->n; b += s->batch_atoms) {
         const int e = std::min(s->n, b + s->batch_atoms);
-        size_t batch_off = 0;
+        size_t batch_off = 0, fp64_off = 0;
         for (int ns = s->na_max / gslot; ns >= 1; --ns) {
             const int key = gslot * ns / 16;
             const bool half = half_ok && (ns & 1) && odd_half(key);
@@ -154,14 +155,26 @@ int prepare_columns(elses_system s) {
                                          : krylov_blocks_per_sm(na, kdeg);
             if (bps < 1) return fail(ELSES_ERR_CAPACITY, "Krylov kernel cannot be resident (%d-atom class)", na);
             // a count fixed by the caller or chosen by the autotuner may use the 4-CTA form
-            const int bps_max = (s->p.krylov_block || half) ? bps : krylov_blocks_per_sm_max(na, kdeg);
+            int bps_max = (s->p.krylov_block || half) ? bps : krylov_blocks_per_sm_max(na, kdeg);
+            int fx = -1;
+            // scratch for the FP64 kernels too: elses_set_hs returns to them without a reallocation
+            fp64_off += (size_t)std::min(count, s->num_sms * bps) * kWarpsPerAtom * 2 * nm * na * 4;
+            if (fx_ok) {
+                const int form = fx_form_for(s->n, s->num_sms);
+                const int nb = fx_blocks_per_sm(form, na, s->max_nb, nm, s->p.reorth != 0, s->p.force_mode == 1);
+                if (nb > 0) {
+                    fx = form;
+                    bps = bps_max = nb;
+                }
+            }
             if (s->p.k3_ctas_per_sm > 0) bps = std::min(bps_max, s->p.k3_ctas_per_sm);
             else if (key < (int)s->tuned_bps.size() && s->tuned_bps[key] > 0) bps = std::min(bps_max, s->tuned_bps[key]);
-            const int grid = std::min(count, s->num_sms * bps);
-            s->k3_launches.push_back({b, e, begin, count, na, grid, bps, half ? 1 : 0, key, batch_off});
+            const int grid = std::min(fx >= 0 ? fx_items(fx, count) : count, s->num_sms * bps);
+            s->k3_launches.push_back({b, e, begin, count, na, grid, bps, half ? 1 : 0, key, fx, batch_off});
             batch_off += s->p.krylov_block ? (size_t)grid * block_krylov_scratch_doubles(nm, na)
+                         : fx >= 0         ? (size_t)grid * fx_scratch_doubles(fx, nm, na)
                                            : (size_t)grid * kWarpsPerAtom * 2 * nm * na * 4;
-            scratch = std::max(scratch, batch_off);
+            scratch = std::max(scratch, fx_ok ? std::max(batch_off, fp64_off) : batch_off);
             if (count > best_items) { best_items = count; s->k3_bps = bps; }
         }
     }
@@ -427,6 +440,12 @@ int ensure_V(elses_system s, cudaStream_t st) {
     return 0;
 }
 
+void launch_krylov(elses_system s, const KrylovArgs& ka, int fx, int grid, int bps, cudaStream_t st) {
+    if (s->p.krylov_block) block_krylov_columns(ka, grid, st);
+    else if (fx >= 0) fx_columns(ka, FxArgs{reinterpret_cast<const int4*>(s->fx_rec.p), s->fx_scale.p, s->skd.Es, s->skd.Ep, 0, 0}, fx, grid, bps, st);
+    else krylov_columns(ka, grid, bps, st);
+}
+
 // Krylov build + projected eigenproblem for atoms [b, e). Writes V and UP either to the stored
 // arrays or to the batch buffers (two-pass), returning the pointers used. form_v false leaves V
 // unformed; in the stored workflow that holds for a batch of every atom (its factors then stay in
@@ -479,8 +498,7 @@ int run_batch(elses_system s, int b, int e, bool stored, double** V_out, int* v_
             CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int), lst));
             ka.queue = q;
         }
-        if (s->p.krylov_block) block_krylov_columns(ka, L.grid, lst);
-        else krylov_columns(ka, L.grid, L.bps, lst);
+        launch_krylov(s, ka, L.fx, L.grid, L.bps, lst);
         s->stats.launches++;
         s->stats.krylov_launches++;
     }
@@ -979,8 +997,17 @@ int elses_build_clusters(elses_system* sys, int n_atoms, const double* pos_dev,
     sk_build(s->pos.p, n, s->box, s->skd, s->row_ptr.p, s->col_idx.p, s->nnzb, s->row_of.p, s->tmap.p,
              s->H.p, s->S.p, s->skr.p, st);
     s->stats.launches += 2;
+    TRY(s->fx_rec.ensure((size_t)s->nnzb * 12));
+    TRY(s->fx_scale.ensure(1));
+    TRY(s->fx_bounds.ensure(6));
+    fx_build(n, s->nnzb, s->row_ptr.p, s->col_idx.p, s->skr.p, s->skd.Es, s->skd.Ep, s->max_nb, s->fx_bounds.p,
+             s->fx_scale.p, s->fx_rec.p, st);
+    s->stats.launches += 3;
+    int fx_ok = 0;
+    CUDA_TRY(cudaMemcpyAsync(&fx_ok, &s->fx_scale.p->ok, sizeof(int), cudaMemcpyDeviceToHost, st));
     if (clusters) TRY(join_side(s, st));   // the cluster lists
     TRY(check_status(s, st));
+    s->fx = fx_ok != 0;
     TRY(prepare_columns(s));
     if (s->p.autotune && s->tuned_bps.empty() && s->p.k3_ctas_per_sm <= 0) TRY(autotune_impl(s, st));
     return ELSES_OK;
@@ -1060,6 +1087,10 @@ int elses_set_hs(elses_system s, int nnzb, const int* row_ptr_dev, const int* co
         TRY(adopt_pattern(s, nnzb, row_ptr_dev, col_idx_dev, st));   // checks before it changes anything
         s->user_hs = true;
         s->drop_graph();
+        TRY(prepare_columns(s));
+    }
+    if (!s->user_hs && s->fx) {   // the launch plan of the FP64 kernels
+        s->user_hs = true;
         TRY(prepare_columns(s));
     }
     s->user_hs = true;

@@ -107,7 +107,12 @@ struct elses_system_s {
     // scratch_off: where the launch's per-CTA scratch starts, so that the class launches of one
     // batch can run at the same time
     // key: the class's bound on cluster size in slots of 16 atoms (its capacity na may be larger)
-    struct K3Launch { int batch_begin, batch_end, item_begin, item_count, na, grid, bps, half, key; size_t scratch_off; };
+    // fx: the form of the fixed-point kernel that runs the class, -1 the FP64 kernels
+    struct K3Launch { int batch_begin, batch_end, item_begin, item_count, na, grid, bps, half, key, fx; size_t scratch_off; };
+    bool fx = false;                       // the fixed-point Krylov form suits the system's H and S
+    DevBuf<elses::FxScale> fx_scale;
+    DevBuf<unsigned long long> fx_bounds;
+    DevBuf<int2> fx_rec;
     cudaStream_t side = nullptr;           // second stream for concurrent class launches
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<K3Launch> k3_launches;
@@ -246,6 +251,7 @@ int prepare_columns(elses_system s);
 int fork_side(elses_system s, cudaStream_t st);
 int join_side(elses_system s, cudaStream_t st);
 KrylovArgs krylov_args(elses_system s, int b, int e);
+void launch_krylov(elses_system s, const KrylovArgs& ka, int fx, int grid, int bps, cudaStream_t st);
 EigArgs eig_args(elses_system s, int b, int e, double* V);
 int ensure_V(elses_system s, cudaStream_t st);
 int reset_archive(elses_system s, cudaStream_t st);
