@@ -210,7 +210,7 @@ struct FxState {
     double2* xd;            // lead: u_n (in units of X), then H u_n or w, in FP64
     const double* skr;      // the FP64 block records
     double Es, Ep;
-    double hh[NC];          // |P|^2
+    double hh[2][NC];       // |P|^2 of the even and the odd steps
     int q[NC], done[NC], nue[NC], we[NC], big[NC];
 };
 
@@ -311,8 +311,10 @@ constexpr int kLead = 3;
 
 template <int T, int kMinB>
 struct FxTmem {
+    // whole groups of four warps share the columns, and an allocation is a power of two
+    static_assert(T % 128 == 0 && (kMinB == 1 || kMinB == 2 || kMinB == 4), "tensor memory split");
     static constexpr int cols = 512 / kMinB;                              // of a CTA
-    static constexpr int units = cols / (T > 128 ? T / 128 : 1) / 4;      // a thread can keep there
+    static constexpr int units = cols / (T / 128) / 4;                     // a thread can keep there
     __device__ static unsigned base(unsigned at) {
         const int warp = threadIdx.x >> 5;
         return at + ((unsigned)(warp & 3) << 21) + (warp >> 2) * (4 * units);
@@ -713,9 +715,22 @@ __device__ __forceinline__ void fx_pass_a(FxState<NC>& st, int n) {
     fx_sweep_y<NC, T>(st, n, 2);
 }
 
-// The scalars of column c after pass A of step n, by one warp: whether u_n exists, its scale, H' and
-// S', and the coefficients of the update. Dot products come in units of 2^60 of the integers'
-// products; u_n = f X, S u_n = f 2^bS Y, H u_n = f 2^bH P.
+// The scalars of column c after pass A of step n, by two warps. Dot products come in units of 2^60 of
+// the integers' products; u_n = f X, S u_n = f 2^bS Y, H u_n = f 2^bH P.
+//
+// X^T S X, and whether u_n exists: the tests on w = 2^we X times the scale of H u_(n-1) (n > 0)
+// against its norm, w^T S w against that of H u_(n-1), both without the common scale. Returns 0, or
+// 1 (no new direction) or 2 (S not positive definite).
+template <int NC>
+__device__ __forceinline__ int fx_norm_test(const KrylovArgs& a, const FxState<NC>& st, int n, int c, double& xsx) {
+    const int nm = st.nm, RC = 3 * nm + 1;
+    xsx = fx_red_get(fx_at<int>(st.v.red) + c * RC + nm + n, NC * RC) * fx_pow2(60 + st.bS[c]);
+    if (n == 0) return 0;
+    const double w2 = xsx * fx_pow2(2 * st.we[c]), bound = a.breakdown_tol * a.breakdown_tol * st.hh[(n - 1) & 1][c];
+    return w2 < -bound ? 2 : w2 > bound ? 0 : 1;
+}
+
+// First warp: S', the coefficients of the update, and the end of the column.
 template <int NC>
 __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st, int n, int c) {
     const int lane = threadIdx.x & 31, nm = st.nm, nu = st.nu, RC = 3 * nm + 1, RS = NC * RC, PK = nm * (nm + 1) / 2;
@@ -725,40 +740,20 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
     const int* rd = red + c * RC;
     double *f = fx_at<double>(st.v.f) + c * nm, *s = fx_at<double>(st.v.s) + c * nm, *h = fx_at<double>(st.v.h) + c * nm;
     const int bH = st.bH[c], bS = st.bS[c];
-    const double xsx = fx_red_get(rd + nm + n, RS) * fx_pow2(60 + bS);   // X^T S X
-    // the tests on w = 2^we X times the scale of H u_(n-1) (n > 0), against its norm:
-    // w^T S w against that of H u_(n-1), both without the common scale
-    bool stop = false;
-    if (n > 0) {
-        const double w2 = xsx * fx_pow2(2 * st.we[c]), bound = a.breakdown_tol * a.breakdown_tol * st.hh[c];
-        if (w2 < -bound) {
-            if (lane == 0) flag(a.status, DEV_NOT_SPD);
-            stop = true;
-        } else if (!(w2 > bound)) {
-            stop = true;
-        }
-    }
-    __syncwarp();
+    double xsx;
+    const int stop = fx_norm_test(a, st, n, c, xsx);
     if (stop) {
         if (lane == 0) {
+            if (stop == 2) flag(a.status, DEV_NOT_SPD);
             st.nue[c] = n;
             st.done[c] = 1;
             atomicSub(&st.live, 1);
         }
     } else {
-        const double fn = rsqrt(xsx);
+        const double fn = rsqrt(xsx), sn = fn * fx_pow2(60 + bS);
         if (lane == 0) {
             f[n] = fn;
-            s[n] = fn * fx_pow2(60 + bS);
-            st.hh[c] = fx_red_get(rd + 3 * nm, RS) * 0x1p60;     // |P|^2
-            fx_at<int>(st.v.ex)[c * nm + n] = bS;
-            fx_at<int>(st.v.ex)[(NC + c) * nm + n] = bH;
-        }
-        if (lane < 3) {   // entry j of X, Y, P
-            const int al = st.alpha0 + c;
-            const int4* w = fx_at<int4>(lane == 0 ? st.v.X : lane == 1 ? st.v.Y : st.v.P);
-            fx_at<int2>(st.v.row)[(lane * NC + c) * nm + n] =
-                reinterpret_cast<const int2*>(w + fx_unit<NC>(st.qJ, al >> 1, c))[al & 1];
+            s[n] = sn;
         }
         double* hess = a.bstore ? a.bstore + (size_t)(4 * st.atom + st.alpha0 + c) * a.bstride + 3 * a.bvec : nullptr;
         if (hess && n > 0 && lane == 0)     // beta_(n-1) = |w|_S
@@ -768,13 +763,10 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
         double* E = fx_at<double>(st.v.E) + (size_t)c * PK;
         const int pk0 = n * (n + 1) / 2;
         bool big = false;
-        const double sn = s[n], pn = fn * fx_pow2(60 + bH);
         for (int k = lane; k <= n; k += 32) {
-            const double fk = f[k];
-            const double spk = fk * (sn * fx_red_get(rd + nm + k, RS));
-            a.Hp[col * PK + pk0 + k] = fk * (pn * fx_red_get(rd + k, RS));
-            a.Sp[col * PK + pk0 + k] = spk;
+            const double spk = f[k] * (sn * fx_red_get(rd + nm + k, RS));
             const double hk = s[k] * fx_red_get(rd + 2 * nm + k, RS);     // SU_k . H u_n over f 2^bH
+            a.Sp[col * PK + pk0 + k] = spk;
             h[k] = hk;
             if (hess) hess[(size_t)n * nm + k] = hk * (fn * fx_pow2(bH));
             if (overlap) {
@@ -798,6 +790,7 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
             double gk[2] = {0.0, 0.0};
             for (int r = 0; r < 2; ++r) {
                 const int k = lane + 32 * r;
+                if (32 * r > n) break;
                 if (k > n) continue;
                 double eh = 0.0;
                 if (overlap && !st.big[c]) {
@@ -825,6 +818,33 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
     }
 }
 
+// Second warp: H', |P|^2, the exponents, and entry j of the vectors.
+template <int NC>
+__device__ __forceinline__ void fx_scalars_h(const KrylovArgs& a, FxState<NC>& st, int n, int c) {
+    const int lane = threadIdx.x & 31, nm = st.nm, RC = 3 * nm + 1, RS = NC * RC, PK = nm * (nm + 1) / 2;
+    const int* rd = fx_at<int>(st.v.red) + c * RC;
+    const int bH = st.bH[c];
+    double xsx;
+    if (fx_norm_test(a, st, n, c, xsx)) return;
+    const double fn = rsqrt(xsx), pn = fn * fx_pow2(60 + bH);
+    const size_t col = (size_t)4 * (st.atom - a.atom_begin) + st.alpha0 + c;
+    for (int k = lane; k <= n; k += 32) {
+        const double fk = k == n ? fn : fx_at<double>(st.v.f)[c * nm + k];
+        a.Hp[col * PK + n * (n + 1) / 2 + k] = fk * (pn * fx_red_get(rd + k, RS));
+    }
+    if (lane == 0) {
+        st.hh[n & 1][c] = fx_red_get(rd + 3 * nm, RS) * 0x1p60;
+        fx_at<int>(st.v.ex)[c * nm + n] = st.bS[c];
+        fx_at<int>(st.v.ex)[(NC + c) * nm + n] = bH;
+    }
+    if (lane < 3) {
+        const int al = st.alpha0 + c;
+        const int4* w = fx_at<int4>(lane == 0 ? st.v.X : lane == 1 ? st.v.Y : st.v.P);
+        fx_at<int2>(st.v.row)[(lane * NC + c) * nm + n] =
+            reinterpret_cast<const int2*>(w + fx_unit<NC>(st.qJ, al >> 1, c))[al & 1];
+    }
+}
+
 // w = P - sum_{k <= n} g_k X_k as 64-bit numbers, into X or in place (into P).
 template <int NC, int T, int kMinB>
 __device__ __forceinline__ void fx_update(FxState<NC>& st, int n, bool into_x, unsigned long long* bits, unsigned* top) {
@@ -837,63 +857,51 @@ __device__ __forceinline__ void fx_update(FxState<NC>& st, int n, bool into_x, u
     unsigned long long mW = 0;
     unsigned mT = 0;
 #pragma unroll 1
-    for (int i0 = 0; i0 < upt; i0 += 3) {
-        Fx acc[6];
+    for (int i0 = 0; i0 < upt; i0 += 2) {
+        Fx acc[4];
         const int ua = min(tid + i0 * T, units - 1), ub = min(tid + (i0 + 1) * T, units - 1);
-        const int uc = min(tid + (i0 + 2) * T, units - 1);
-        int k = 0;
+        // vectors at to at + 3: w[kk], w[4 + kk] the two units of vector at + kk
+        auto apply = [&](int at, int kend, const int4 (&w)[8]) {
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const int2 gk = at + kk < kend ? g[at + kk] : make_int2(0, 0);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    fx_mac(acc[2 * i], gk, fx_lo(w[4 * i + kk]));
+                    fx_mac(acc[2 * i + 1], gk, fx_hi(w[4 * i + kk]));
+                }
+            }
+        };
 #pragma unroll 1
-        for (; k < kT && k <= n; k += 2) {
-            int4 w[6];
-            fx_tmem_ld3x2(tm + 4 * (k * upt + i0), 4 * upt, w);
-            const int2 ga = g[k], gb = k < n ? g[k + 1] : make_int2(0, 0);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                fx_mac(acc[2 * i], ga, fx_lo(w[i]));
-                fx_mac(acc[2 * i + 1], ga, fx_hi(w[i]));
-            }
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                fx_mac(acc[2 * i], gb, fx_lo(w[3 + i]));
-                fx_mac(acc[2 * i + 1], gb, fx_hi(w[3 + i]));
-            }
+        for (int k = 0; k < kT && k <= n; k += 4) {
+            int4 w[8];
+            fx_tmem_ld4x2(tm + 4 * (k * upt + i0), 4 * upt, w);
+            apply(k, n + 1, w);
         }
-        auto sweep = [&](const int4* base, int k, int kend) {   // vectors k to kend - 1 at base, two at a time
-            const int4* q = base;
-            auto load = [&](int4 (&w)[6]) {   // past the end: the last vector again
+        auto sweep = [&](const int4* base, int k, int kend) {   // vectors k to kend - 1 at base
+            const int4 *q = base, *const last = base + (size_t)(kend - 1 - k) * units;
+            auto load = [&](int4 (&w)[8]) {   // past the end: the last vector again
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    w[3 * kk] = q[ua];
-                    w[3 * kk + 1] = q[ub];
-                    w[3 * kk + 2] = q[uc];
-                    if (q < base + (size_t)(kend - 1 - k) * units) q += units;
+                for (int kk = 0; kk < 4; ++kk) {
+                    w[kk] = q[ua];
+                    w[4 + kk] = q[ub];
+                    if (q < last) q += units;
                 }
             };
-            auto apply = [&](int at, const int4 (&w)[6]) {
-#pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    const int2 gk = at + kk < kend ? g[at + kk] : make_int2(0, 0);
-#pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        fx_mac(acc[2 * i], gk, fx_lo(w[3 * kk + i]));
-                        fx_mac(acc[2 * i + 1], gk, fx_hi(w[3 * kk + i]));
-                    }
-                }
-            };
-            int4 wa[6], wb[6];
+            int4 wa[8], wb[8];
             load(wa);
 #pragma unroll 1
-            for (int at = k; at < kend; at += 4) {
+            for (int at = k; at < kend; at += 8) {
                 load(wb);
-                apply(at, wa);
+                apply(at, kend, wa);
                 load(wa);
-                apply(at + 2, wb);
+                if (at + 4 < kend) apply(at + 4, kend, wb);
             }
         };
         if (n >= kT) sweep(fx_at<int4>(st.v.cache), kT, min(kS, n + 1));
         if (n >= kS) sweep(st.gU + (size_t)kS * units, kS, n + 1);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
+        for (int i = 0; i < 2; ++i) {
             const int u = tid + (i0 + i) * T;
             if (i0 + i < upt && u < units) {
                 if (n < kLead) {
@@ -1189,8 +1197,8 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
                 st.units = units;
                 st.upt = upt;
                 st.nu = nu;
-                // (the update reads up to two units past a vector in tensor memory)
-                st.kT = min((Tm::units - 2) / upt, nu) & ~3;
+                // (the update reads up to one unit past a vector in tensor memory)
+                st.kT = min((Tm::units - 1) / upt, nu) & ~3;
                 st.kS = st.kT + min(nu - st.kT, vecs);
                 st.kY = min(nu, vecs - (st.kS - st.kT));
                 // xd: the last vector's place in shared memory while that is free, else scratch
@@ -1219,8 +1227,11 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
                 __syncthreads();
                 fx_take_products<NC, T>(st, n);
                 fx_pass_a<NC, T, kMinB>(st, n);
+                const int warp = threadIdx.x >> 5;
+                const bool idle = warp >= 2 * NC || st.done[warp % NC];   // (done changes below)
                 __syncthreads();
-                if (threadIdx.x < 32 * NC && !st.done[threadIdx.x >> 5]) fx_scalars<NC>(a, st, n, threadIdx.x >> 5);
+                if (!idle && warp < NC) fx_scalars<NC>(a, st, n, warp);
+                else if (!idle) fx_scalars_h<NC>(a, st, n, warp - NC);
                 __syncthreads();
                 if (a.bstore) {
                     fx_keep_step<NC, T>(a, st, n);

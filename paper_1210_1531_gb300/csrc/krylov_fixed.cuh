@@ -71,7 +71,8 @@ __device__ __forceinline__ void fx_coefs(const double (&gk)[2], int n, int2* g, 
     const int e = max((int)(top >> 20) - 1023, -900);           // largest |g| < 2^(e + 1)
     // the sum over 2^e, in single precision and rounded up
     const double down = __longlong_as_double((long long)(1023 - e) << 52);
-    float sum = __double2float_ru(fabs(gk[0]) * down) + __double2float_ru(fabs(gk[1]) * down);
+    float sum = __double2float_ru(fabs(gk[0]) * down);
+    if (n >= 32) sum += __double2float_ru(fabs(gk[1]) * down);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     const int es = (int)(__float_as_uint(sum * 1.001f) >> 23) - 127 + 1;      // sum < 2^(e + es)
@@ -79,7 +80,7 @@ __device__ __forceinline__ void fx_coefs(const double (&gk)[2], int n, int2* g, 
     const double scale = __longlong_as_double((long long)(1023 + eg) << 52);
 #pragma unroll
     for (int r = 0; r < 2; ++r)
-        if (lane + 32 * r <= n) g[lane + 32 * r] = fx_split(__double2ll_rn(gk[r] * scale));
+        if (32 * r <= n && lane + 32 * r <= n) g[lane + 32 * r] = fx_split(__double2ll_rn(gk[r] * scale));
     if (lane == 0) *shift = 56 - eg;
 }
 
@@ -120,14 +121,16 @@ __device__ __forceinline__ void fx_tmem_ld(unsigned at, int step, int4 (&v)[N]) 
                      : FX_OUT(v[0]), FX_OUT(v[1]), FX_OUT(v[2]), FX_OUT(v[3])
                      : "r"(at), "r"(at + step), "r"(at + 2 * step), "r"(at + 3 * step) : "memory");
 }
-// three neighbouring units of two vectors `step` columns apart
-__device__ __forceinline__ void fx_tmem_ld3x2(unsigned at, int step, int4 (&v)[6]) {
+// two neighbouring units of four vectors `step` columns apart: v[kk], v[4 + kk] of vector kk
+__device__ __forceinline__ void fx_tmem_ld4x2(unsigned at, int step, int4 (&v)[8]) {
     __syncwarp();
-    asm volatile(FX_LD(0, 1, 2, 3, 24) FX_LD(4, 5, 6, 7, 25) FX_LD(8, 9, 10, 11, 26)
-                 FX_LD(12, 13, 14, 15, 27) FX_LD(16, 17, 18, 19, 28) FX_LD(20, 21, 22, 23, 29)
+    asm volatile(FX_LD(0, 1, 2, 3, 32) FX_LD(4, 5, 6, 7, 33) FX_LD(8, 9, 10, 11, 34) FX_LD(12, 13, 14, 15, 35)
+                 FX_LD(16, 17, 18, 19, 36) FX_LD(20, 21, 22, 23, 37) FX_LD(24, 25, 26, 27, 38) FX_LD(28, 29, 30, 31, 39)
                  "tcgen05.wait::ld.sync.aligned;"
-                 : FX_OUT(v[0]), FX_OUT(v[1]), FX_OUT(v[2]), FX_OUT(v[3]), FX_OUT(v[4]), FX_OUT(v[5])
-                 : "r"(at), "r"(at + 4), "r"(at + 8), "r"(at + step), "r"(at + step + 4), "r"(at + step + 8) : "memory");
+                 : FX_OUT(v[0]), FX_OUT(v[1]), FX_OUT(v[2]), FX_OUT(v[3]), FX_OUT(v[4]), FX_OUT(v[5]), FX_OUT(v[6]),
+                   FX_OUT(v[7])
+                 : "r"(at), "r"(at + step), "r"(at + 2 * step), "r"(at + 3 * step), "r"(at + 4), "r"(at + step + 4),
+                   "r"(at + 2 * step + 4), "r"(at + 3 * step + 4) : "memory");
 }
 #undef FX_LD
 #undef FX_OUT
