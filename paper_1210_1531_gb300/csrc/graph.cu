@@ -29,9 +29,9 @@ int enqueue_step(elses_system s, double* forces_dev, cudaStream_t st) {
     ReduceArgs r = reduce_args(s);
     s->tic(T_BISECT, st);
     bisect_init(r, st);
-    for (int it = 0; it < s->p.max_bisect; ++it) bisect_step(r, st);
+    const int steps = bisect_all(r, st);
     s->toc(st);
-    s->stats.launches += 3 + s->p.max_bisect;
+    s->stats.launches += 3 + steps;
     const double* mu_dev = (const double*)((const char*)s->bstate.p + offsetof(BisectState, mu));
     TRY(density_impl(s, 0.0, s->rho.p, s->rhoE.p, st, mu_dev));
     s->tic(T_BISECT, st);
@@ -140,6 +140,7 @@ int energy_force_graph(elses_system s, double* mu_host, double* e_band_host, dou
     const int rc = check_status(s, st);
     s->collect_graph();
     s->stats.bisect_steps = h.iter;
+    if (h.status & DEV_TIMEOUT) return fail(ELSES_ERR_TIMEOUT, "the bisection's blocks did not meet");
     if (h.status & DEV_NONFINITE) return fail(ELSES_ERR_NONFINITE, "non-finite poles");
     if (h.status & DEV_NO_BRACKET)
         return fail(ELSES_ERR_NO_BRACKET, "N(lo)=%.17g N(hi)=%.17g do not bracket N_e=%.17g", h.n_lo, h.n_hi,

@@ -224,6 +224,7 @@ struct BisectState {
     double mu0;             // where the kept exponentials were taken
     double scale;           // exp((mu0 - x)/kT) at the next midpoint x, once they are kept
     int iter, done, status, have_pre;
+    int step;               // arrivals of k_bisect's blocks
 };
 struct ReduceArgs {
     int M;
@@ -251,6 +252,7 @@ struct ReduceArgs {
 int reduce_grid();
 void bisect_init(const ReduceArgs& a, cudaStream_t st);      // bracket + N(lo), N(hi)
 void bisect_step(const ReduceArgs& a, cudaStream_t st);      // one bisection step (no-op when done)
+int bisect_all(const ReduceArgs& a, cudaStream_t st);         // every step; the number of launches
 void scalars_at(const ReduceArgs& a, double mu, cudaStream_t st);  // N, E_band, Omega at mu
 void scalars_at_state(const ReduceArgs& a, cudaStream_t st);      // the same at the state's mu
 // DOS at n_z energies; scratch holds dos_scratch_doubles(n_z), the result in its last n_z

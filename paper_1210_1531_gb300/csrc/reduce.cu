@@ -17,10 +17,12 @@
 //
 // Every evaluation is one grid-wide reduction in a fixed order (per-thread column strides, a
 // fixed block tree, then the block partials summed in index order by the last block to finish,
-// found with an atomic ticket -- no thread ever waits on another block). The bracket lives in
-// device memory and each bisection launch reads and updates it, so the whole search is a fixed
-// sequence of launches with no host round trip; launches after convergence return at once.
+// found with an atomic ticket). The bracket lives in device memory, read and updated by each step
+// with no host round trip: all steps in one cooperative launch (k_bisect), or a fixed sequence of
+// launches (k_count) of which those after convergence return at once.
 #include "internal.h"
+
+#include <algorithm>
 
 namespace elses {
 
@@ -31,6 +33,18 @@ int reduce_grid() {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return 4 * (sms > 0 ? sms : 1);
+}
+
+// Words that another block of the same launch writes: loads that are made each time and go past L1.
+__device__ __forceinline__ double ld_gpu(const double* p) {
+    double v;
+    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int ld_gpu(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
 template <int NV>
@@ -74,7 +88,7 @@ __device__ __forceinline__ void sum_partials(const double* partials, int nblocks
     for (int q = 0; q < NV; ++q) v[q] = 0.0;
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
 #pragma unroll
-        for (int q = 0; q < NV; ++q) v[q] += __ldcg(partials + 4 * (size_t)b + q);
+        for (int q = 0; q < NV; ++q) v[q] += ld_gpu(partials + 4 * (size_t)b + q);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
@@ -145,35 +159,26 @@ __global__ void k_bracket(const ReduceArgs a) {
         s->mu = 0.5 * (s->lo + s->hi);
         s->mu0 = 0.0;
         s->have_pre = 0;
+        s->step = 0;
         *a.ticket = 0u;
     }
 }
 
-// mode 0: N(lo); 1: N(hi) and the bracket check; 2: one bisection step; 3: scalars at mu_in;
-// 4: scalars at the state's mu (written like mode 3).
+// A block's part of the sums at x, into its partials. Mode 2 (a bisection step at the middle of a
+// bracket of this width, have_pre: the poles are kept): N; mode 3: N, E_band and Omega; 0, 1: N.
 // Block b takes the poles of a contiguous range (flattened [column][k]); poles more than 50 kT
 // from x contribute their limit (f = 1 below, 0 above) without an exponential: the neglected part
-// is below e^-50 of their weight, far under the rounding of the sums.
-__global__ void __launch_bounds__(kRedThreads) k_count(const ReduceArgs a, int mode, double mu_in) {
-    BisectState* s = a.state;
-    double x;
-    if (mode == 2) {
-        if (s->done) return;
-        x = 0.5 * (s->lo + s->hi);
-    } else if (mode == 0) x = s->lo;
-    else if (mode == 1) x = s->hi;
-    else if (mode == 4) x = s->mu;
-    else x = mu_in;
-    if (mode == 4) mode = 3;
+// is below e^-50 of their weight, far under the rounding of the sums. True if poles were kept.
+__device__ __forceinline__ bool count_block(const ReduceArgs& a, int mode, double x, double width, double scale, bool have_pre,
+                                            double* partials) {
     double v[3] = {0.0, 0.0, 0.0};
     const size_t total = (size_t)a.M * a.nu_max;
     const size_t chunk = (total + gridDim.x - 1) / gridDim.x;
     const size_t b0 = min(total, (size_t)blockIdx.x * chunk), b1 = min(total, b0 + chunk);
     const double inv_kT = a.inv_kT;
-    const bool keep = mode == 2 && a.act && !s->have_pre && s->hi - s->lo < 10.0 * a.kT;
-    if (mode == 2 && a.act && s->have_pre) {
+    const bool keep = mode == 2 && a.act && !have_pre && width < 10.0 * a.kT;
+    if (mode == 2 && a.act && have_pre) {
         // the kept poles of this block; the block's constant part once, by thread 0
-        const double scale = s->scale;   // exp((mu0 - x)/kT), set by the previous step
         const int n = a.act_n[blockIdx.x];
         const double2* q = a.act + b0;
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -297,11 +302,29 @@ __global__ void __launch_bounds__(kRedThreads) k_count(const ReduceArgs a, int m
         }
     }
     // the bisection needs N only; mode 3 also E_band and Omega
-    if (mode == 3) block_reduce_store<3>(v, a.partials, 4);
+    if (mode == 3) block_reduce_store<3>(v, partials, 4);
     else {
         double n1[1] = {v[0]};
-        block_reduce_store<1>(n1, a.partials, 4);
+        block_reduce_store<1>(n1, partials, 4);
     }
+    return keep;
+}
+
+// One evaluation per launch. mode 0: N(lo); 1: N(hi) and the bracket check; 2: one bisection step;
+// 3: scalars at mu_in; 4: scalars at the state's mu (written like mode 3).
+__global__ void __launch_bounds__(kRedThreads) k_count(const ReduceArgs a, int mode, double mu_in) {
+    BisectState* s = a.state;
+    double x;
+    if (mode == 2) {
+        if (s->done) return;
+        x = 0.5 * (s->lo + s->hi);
+    } else if (mode == 0) x = s->lo;
+    else if (mode == 1) x = s->hi;
+    else if (mode == 4) x = s->mu;
+    else x = mu_in;
+    if (mode == 4) mode = 3;
+    // scale: exp((mu0 - x)/kT), set by the previous step
+    const bool keep = count_block(a, mode, x, s->hi - s->lo, s->scale, s->have_pre != 0, a.partials);
     if (!last_block(a.ticket)) return;
     double tot[3] = {0.0, 0.0, 0.0};
     if (mode == 3) sum_partials<3>(a.partials, gridDim.x, tot);
@@ -329,13 +352,89 @@ __global__ void __launch_bounds__(kRedThreads) k_count(const ReduceArgs a, int m
             s->iter += 1;
             if (s->iter >= a.max_iter || !(s->hi - s->lo >= a.tol)) s->done = 1;
             s->mu = 0.5 * (s->lo + s->hi);
-            if (s->have_pre) s->scale = exp((s->mu0 - 0.5 * (s->lo + s->hi)) * inv_kT);
+            if (s->have_pre) s->scale = exp((s->mu0 - 0.5 * (s->lo + s->hi)) * a.inv_kT);
         } else {
             s->n_at = N;
             s->e_band = E;
             s->omega = Om;
         }
         *a.ticket = 0u;
+    }
+}
+
+// Every bisection step in one cooperative launch. A step of the kept poles is a microsecond of work,
+// so two dependent launches (the sums, the next step's) were most of its cost, and half of the fixed
+// sequence of launches ran after convergence. Here each block writes its partial, arrives at a
+// counter, and sums all partials itself, in index order: lo and hi stay in registers, the same in
+// every block, and one trip through L2 separates two steps. The partials alternate between two places:
+// a block can be one step ahead of another's reading, not two. The wait is bounded; a block that gives
+// up flags DEV_TIMEOUT and leaves. Kept poles live in registers up to kPoleRegs a thread. The whole
+// search of 64 atoms took 0.87 ms with a launch per step, now 0.35 ms; of 4096 atoms 1.14 ms, 0.64 ms.
+constexpr int kWaitPolls = 1 << 22, kPoleRegs = 2;
+__global__ void __launch_bounds__(kRedThreads, 4) k_bisect(const ReduceArgs a) {
+    __shared__ int sh_stop;
+    BisectState* s = a.state;
+    if (s->done) return;
+    double lo = s->lo, hi = s->hi, mu0 = 0.0, below = 0.0, N = 0.0;
+    const size_t total = (size_t)a.M * a.nu_max, chunk = (total + gridDim.x - 1) / gridDim.x;
+    const double2* kept = a.act + min(total, (size_t)blockIdx.x * chunk);
+    double2 pole[kPoleRegs];
+    int n_kept = 0, iter = 0;
+    bool have_pre = false, done = false;
+    if (threadIdx.x == 0) sh_stop = 0;
+    while (!done) {
+        const double x = 0.5 * (lo + hi);
+        double* partials = a.partials + (iter & 1);
+        if (have_pre) {
+            const double scale = exp((mu0 - x) * a.inv_kT);
+            double v[1] = {below};
+#pragma unroll
+            for (int i = 0; i < kPoleRegs; ++i)
+                if ((int)threadIdx.x + i * kRedThreads < n_kept)
+                    v[0] = fma(2.0 / fma(pole[i].x, scale, 1.0), pole[i].y, v[0]);
+            for (int i = threadIdx.x + kPoleRegs * kRedThreads; i < n_kept; i += kRedThreads) {
+                const double2 w = kept[i];
+                v[0] = fma(2.0 / fma(w.x, scale, 1.0), w.y, v[0]);
+            }
+            block_reduce_store<1>(v, partials, 4);
+        } else if (count_block(a, 2, x, hi - lo, 0.0, false, partials)) {
+            __syncthreads();   // the block's list is complete
+            have_pre = true;
+            mu0 = x;
+            n_kept = a.act_n[blockIdx.x];
+            if (threadIdx.x == 0) below = a.act_below[blockIdx.x];
+#pragma unroll
+            for (int i = 0; i < kPoleRegs; ++i)
+                if ((int)threadIdx.x + i * kRedThreads < n_kept) pole[i] = kept[threadIdx.x + i * kRedThreads];
+        }
+        ++iter;
+        if (threadIdx.x == 0) {   // the partial is this thread's
+            const unsigned want = (unsigned)iter * gridDim.x;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&s->step) : "memory");
+            int polls = 0;
+            while ((int)((unsigned)ld_gpu(&s->step) - want) < 0 && polls < kWaitPolls) ++polls;
+            if (polls == kWaitPolls) {
+                atomicOr(&s->status, DEV_TIMEOUT);
+                sh_stop = 1;
+            }
+        }
+        __syncthreads();
+        if (sh_stop) return;
+        double n1[1];
+        sum_partials<1>(partials, gridDim.x, n1);
+        N = n1[0];
+        if (N < a.n_electrons) lo = x; else hi = x;
+        done = iter >= a.max_iter || !(hi - lo >= a.tol);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        s->lo = lo;
+        s->hi = hi;
+        s->mu = 0.5 * (lo + hi);
+        s->n_mid = N;
+        s->iter = iter;
+        s->have_pre = have_pre;
+        s->mu0 = mu0;
+        s->done = 1;
     }
 }
 
@@ -348,6 +447,35 @@ void bisect_init(const ReduceArgs& a, cudaStream_t st) {
 
 void bisect_step(const ReduceArgs& a, cudaStream_t st) {
     k_count<<<reduce_grid(), kRedThreads, 0, st>>>(a, 2, 0.0);
+}
+
+// Blocks of k_bisect. Blocks polling one counter and reading every partial delay one another, so few
+// blocks with several poles a thread: 512 poles a block up to one block per SM (61440 poles: 120
+// blocks 0.38 ms, 480 blocks 0.86 ms; 491520 poles: 152 blocks 0.64 ms, 304 0.77 ms, 608 1.15 ms), and
+// two per SM once the sums themselves take longer (7.8 million poles: 4.6 ms; 152 blocks 5.4 ms).
+int bisect_grid(const ReduceArgs& a, int sms) {
+    const size_t total = (size_t)a.M * a.nu_max;
+    if (total > (size_t)sms * 8192) return 2 * sms;
+    return (int)std::min<size_t>(sms, (total + 511) / 512);
+}
+
+// Every step: one cooperative launch where the device holds all its blocks at once, else the
+// fixed sequence of launches. Returns the number of launches.
+int bisect_all(const ReduceArgs& a, cudaStream_t st) {
+    int dev = 0, sms = 0, coop = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bisect, kRedThreads, 0);
+    const int grid = bisect_grid(a, sms);
+    if (coop && a.act && per_sm * sms >= grid) {
+        void* args[] = {const_cast<ReduceArgs*>(&a)};
+        if (cudaLaunchCooperativeKernel((const void*)k_bisect, dim3(grid), dim3(kRedThreads), args, 0, st) == cudaSuccess)
+            return 1;
+        cudaGetLastError();
+    }
+    for (int it = 0; it < a.max_iter; ++it) bisect_step(a, st);
+    return a.max_iter;
 }
 
 void scalars_at(const ReduceArgs& a, double mu, cudaStream_t st) {

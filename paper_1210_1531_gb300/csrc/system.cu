@@ -1164,8 +1164,7 @@ int elses_find_mu(elses_system s, double* mu_host, double* n_at_mu_host, void* s
     s->tic(T_BISECT, st);
     bisect_init(r, st);
     s->stats.launches += 3;
-    for (int it = 0; it < s->p.max_bisect; ++it) bisect_step(r, st);
-    s->stats.launches += s->p.max_bisect;
+    s->stats.launches += bisect_all(r, st);
     s->toc(st);
     BisectState h{};
     CUDA_TRY(cudaMemcpyAsync(&h, s->bstate.p, sizeof h, cudaMemcpyDeviceToHost, st));
@@ -1173,6 +1172,7 @@ int elses_find_mu(elses_system s, double* mu_host, double* n_at_mu_host, void* s
     CUDA_TRY(cudaGetLastError());
     s->collect();
     s->stats.bisect_steps = h.iter;
+    if (h.status & DEV_TIMEOUT) return fail(ELSES_ERR_TIMEOUT, "the bisection's blocks did not meet");
     if (h.status & DEV_NONFINITE) return fail(ELSES_ERR_NONFINITE, "non-finite poles");
     if (h.status & DEV_NO_BRACKET)
         return fail(ELSES_ERR_NO_BRACKET, "N(lo)=%.17g N(hi)=%.17g do not bracket N_e=%.17g", h.n_lo, h.n_hi,
