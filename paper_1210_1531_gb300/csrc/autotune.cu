@@ -20,6 +20,7 @@ int autotune_impl(elses_system s, cudaStream_t st) {
     const int nm = s->nu_max;
     const int kdeg = s->user_hs ? s->max_nb : s->deg_cap;
     s->tuned_bps.assign(s->na_max / 16 + 1, 0);
+    s->tuned_fx.assign(s->na_max / 16 + 1, 0);
     s->tuned_order.assign(s->na_max / 16 + 1, 0);
     s->tuned_half.assign(s->na_max / 16 + 1, 0);
     const bool half_ok = s->p.k3_lanes != 32 && s->p.force_mode == 0 && !s->p.krylov_block;
@@ -46,21 +47,22 @@ int autotune_impl(elses_system s, cudaStream_t st) {
     for (const auto& L : launches) {
         if (rc || seen[L.key]) continue;   // each class once, at its first batch
         seen[L.key] = 1;
+        const int fx = s->user_hs ? -1 : L.fx;
         const int ns = L.key;
         // the kernel forms to compare: a class of an odd number of 16-atom slots runs either
         // with half-warps (capacity 16 ns) or with whole warps (capacity 16 (ns + 1))
         struct Form { int half, na, maxb; };
         std::vector<Form> forms;
-        if (half_ok && (ns & 1) && L.fx < 0) forms = {{1, 16 * ns, 0}, {0, 16 * (ns + 1), 0}};
+        if (half_ok && (ns & 1) && fx < 0) forms = {{1, 16 * ns, 0}, {0, 16 * (ns + 1), 0}};
         else forms = {{L.half, L.na, 0}};
         int maxb_all = 0;
         for (auto& f : forms) {
-            f.maxb = L.fx >= 0         ? fx_blocks_per_sm(L.fx, f.na, s->max_nb, nm, s->p.reorth != 0, s->p.force_mode == 1)
+            f.maxb = fx >= 0         ? fx_blocks_per_sm(fx, f.na, s->max_nb + 1, nm, s->p.reorth != 0, s->p.force_mode == 1)
                      : s->p.krylov_block ? block_krylov_blocks_per_sm(f.na, kdeg)
                      : f.half          ? krylov_half_blocks_per_sm(f.na, kdeg)
                                        : krylov_blocks_per_sm_max(f.na, kdeg);
             maxb_all = std::max(maxb_all, f.maxb);
-            const size_t per_cta = L.fx >= 0         ? fx_scratch_doubles(L.fx, nm, f.na)
+            const size_t per_cta = fx >= 0         ? fx_scratch_doubles(fx, nm, f.na)
                                    : s->p.krylov_block ? block_krylov_scratch_doubles(nm, f.na)
                                                      : (size_t)kWarpsPerAtom * 2 * nm * f.na * 4;
             if ((rc = s->kscratch.ensure((size_t)s->num_sms * f.maxb * per_cta)) < 0) break;
@@ -81,7 +83,7 @@ int autotune_impl(elses_system s, cudaStream_t st) {
             ka.order = s->order.p + L.item_begin;
             ka.n_items = sample;
             ka.scratch = s->kscratch.p;
-            const int grid = std::min(L.fx >= 0 ? fx_items(L.fx, sample) : sample, s->num_sms * b);
+            const int grid = std::min(fx >= 0 ? fx_items(fx, sample) : sample, s->num_sms * b);
             float ms = 0.f;
             for (int rep = 0; rep < 2; ++rep) {       // the first launch warms caches and clocks
                 if (s->p.schedule == 1) {
@@ -89,7 +91,7 @@ int autotune_impl(elses_system s, cudaStream_t st) {
                     if (cudaMemsetAsync(ka.queue, 0, sizeof(int), st) != cudaSuccess) { rc = fail(ELSES_ERR_CUDA, "memset"); break; }
                 }
                 cudaEventRecord(e0, st);
-                launch_krylov(s, ka, L.fx, grid, b, st);
+                launch_krylov(s, ka, fx, grid, b, st);
                 cudaEventRecord(e1, st);
                 s->stats.launches++;
             }
@@ -104,7 +106,10 @@ int autotune_impl(elses_system s, cudaStream_t st) {
         }
         if (!rc && forms.size() == 2) s->tuned_half[ns] = forms[best_f].half ? 1 : 2;
         const int chosen_na = forms[best_f].na, chosen_half = forms[best_f].half;
-        if (!rc) s->tuned_bps[ns] = best_b;
+        if (!rc) {
+            s->tuned_bps[ns] = best_b;
+            s->tuned_fx[ns] = fx >= 0;
+        }
         if (rc || s->p.schedule != 1 || L.item_count < 4 * s->num_sms * best_b) continue;
         // queue order of the whole class: as planned (decreasing cluster size), then atom order
         std::vector<int> seg(L.item_count);
@@ -126,11 +131,11 @@ int autotune_impl(elses_system s, cudaStream_t st) {
             ka.n_items = L.item_count;
             ka.scratch = s->kscratch.p;
             ka.queue = s->counters.p + kQueue0;
-            const int grid = std::min(L.fx >= 0 ? fx_items(L.fx, L.item_count) : L.item_count, s->num_sms * best_b);
+            const int grid = std::min(fx >= 0 ? fx_items(fx, L.item_count) : L.item_count, s->num_sms * best_b);
             for (int rep = 0; rep < 2; ++rep) {
                 cudaMemsetAsync(ka.queue, 0, sizeof(int), st);
                 cudaEventRecord(e0, st);
-                launch_krylov(s, ka, L.fx, grid, best_b, st);
+                launch_krylov(s, ka, fx, grid, best_b, st);
                 cudaEventRecord(e1, st);
                 s->stats.launches++;
             }

@@ -59,7 +59,7 @@ int enqueue_step(elses_system s, double* forces_dev, cudaStream_t st) {
 // forces output, the parameters and the Krylov launch plan.
 std::vector<long long> graph_key(elses_system s, const double* forces_dev) {
     std::vector<long long> k = {(long long)g_alloc_epoch, (long long)(uintptr_t)forces_dev, s->n, s->nnzb,
-                                s->nu_max, s->na_max, s->batch_atoms, s->user_hs ? 1 : 0, s->max_nb,
+                                s->nu_max, s->na_max, s->batch_atoms, s->user_hs ? 1 + (s->fx_user ? 1 : 0) : 0, s->max_nb,
                                 s->max_cl, s->deg_cap};
     auto add_bytes = [&k](const void* src, size_t bytes) {
         std::vector<long long> w((bytes + 7) / 8, 0);
@@ -71,7 +71,7 @@ std::vector<long long> graph_key(elses_system s, const double* forces_dev) {
     add_bytes(&s->skd, sizeof(s->skd));
     for (int b = 0; b < s->n; b += s->batch_atoms) k.push_back(s->h_row_ptr[b]);   // batch pattern offsets
     for (const auto& L : s->k3_launches) {
-        k.insert(k.end(), {L.batch_begin, L.batch_end, L.item_begin, L.item_count, L.na, L.grid, L.bps, L.fx,
+        k.insert(k.end(), {L.batch_begin, L.batch_end, L.item_begin, L.item_count, L.na, L.grid, L.bps, L.fx, L.fx_dense, L.grid64, L.bps64,
                            (long long)L.scratch_off});
     }
     return k;

@@ -75,6 +75,7 @@ struct KrylovArgs {
     int atom_begin, atom_end;
     const int* order;       // atoms of this launch in processing order (n_items of them)
     int n_items;
+    const int* skip;        // FP64 kernels: nothing to do where this (device) is set and not zero
     int* queue;             // optional: work counter of the persistent queue (batched form)
     int nu_max;             // allocation stride of per-column Krylov arrays
     int nu_default;
@@ -131,6 +132,8 @@ struct AdjointArgs {
 // six words), then the launch of a size class
 void fx_build(int n, int nnzb, const int* row_ptr, const int* col_idx, const double* skr, double Es, double Ep,
               int max_row, unsigned long long* bounds, FxScale* scale, int2* rec, cudaStream_t st);
+void fx_build_dense(int n, int nnzb, const int* row_ptr, const double* H, const double* S, int max_row,
+                    unsigned long long* bounds, FxScale* scale, int2* rec, cudaStream_t st);
 int fx_form_for(int n, int sms);                       // for a system of n atoms
 int fx_items(int form, int count);                     // CTAs' work items of it
 int fx_blocks_per_sm(int form, int na, int max_row, int nu, bool overlap, bool store);   // 0: the class does not fit

@@ -47,6 +47,7 @@ size_t krylov_smem_bytes(int na_max, int deg_max) {
 template <bool kStore, int kMinB>
 __global__ void __launch_bounds__(kThreads, kMinB) k_krylov(const KrylovArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (a.skip && *a.skip) return;
     const int NA = a.na_max;
     double* vec = reinterpret_cast<double*>(smem_raw);
     double* hbuf = vec + (size_t)kWarpsPerAtom * 2 * NA * 4;
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(kThreads, kMinB) k_krylov(const KrylovArgs a) 
 constexpr int kHalfThreads = 16 * kWarpsPerAtom;
 __global__ void __launch_bounds__(kHalfThreads, 6) k_krylov_half(const KrylovArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (a.skip && *a.skip) return;
     const int NA = a.na_max;
     double* vec = reinterpret_cast<double*>(smem_raw);
     double* hbuf = vec + (size_t)kWarpsPerAtom * 2 * NA * 4;

@@ -1,6 +1,6 @@
-// a3 + a4 in 57-bit fixed point on the integer pipe: the per-column Krylov build of krylov.cu for
-// Slater-Koster systems, the same recursion (krylov.cu's header) on vectors held as integers with
-// one power-of-two scale each.
+// a3 + a4 in 57-bit fixed point on the integer pipe: the per-column Krylov build of krylov.cu,
+// the same recursion (krylov.cu's header) on vectors held as integers with one power-of-two scale
+// each, for Slater-Koster systems and for a caller's H and S.
 //
 // Why integers: the FP64 pipe of this chip retires 1.68 FMA per clock and SM, and the FP64 form of
 // the recursion keeps it 92% busy, so no layout makes that form faster. The 32 x 32 + 64-bit integer
@@ -19,14 +19,20 @@
 //
 // Coefficients of the two-centre blocks carry one power-of-two scale per matrix (FxScale): the
 // largest is below 2^57 and the sum of any row's bounds below 2^62 (2^60 for rows of 33 to 64
-// blocks, whose cross terms add up further), so no sum of a sparse product overflows. The host uses
-// this form only where every row sum lies within 2^8 of the largest, so that each row keeps at least
-// the relative precision FP64 gives it.
+// blocks, whose cross terms add up further), so no sum of a sparse product overflows. This form is
+// used only where every row sum lies within 2^8 of the largest, so that each row keeps at least
+// the relative precision FP64 gives it. A caller's dense blocks are held alike, by exact row sums, up
+// to 32 blocks a row: four products a row and block.
+//
+// The host reads whether the form suits a Slater-Koster system when it is built. elses_set_hs does not
+// wait for the device, so with a caller's matrices both kernels are launched and the device decides:
+// the one that is not to run returns at once.
 //
 // Against an 80-bit recursion (48 columns of 512-atom systems, G at three energies, geometric mean
 // of the relative errors; FP64 kernel first): displaced diamond 7.7e-15 / 7.8e-15 with two classical
 // passes and 8.7e-15 / 7.3e-15 with the second from S'; dense disordered carbon 1.11e-14 / 1.06e-14
-// and 1.19e-14 / 1.20e-14.
+// and 1.19e-14 / 1.20e-14; the same H and S as a caller's: 8.3e-15 / 8.5e-15, 7.9e-15 / 7.1e-15,
+// 1.12e-14 / 1.04e-14, 1.04e-14 / 1.06e-14.
 #include <algorithm>
 
 #include "krylov.cuh"
@@ -77,18 +83,20 @@ __global__ void k_fx_bounds(int n, const int* __restrict__ row_ptr, const int* _
 __device__ __forceinline__ long long fx_round(double v, int e) { return llrint(ldexp(v, e)); }
 
 // The scales, and whether the fixed-point form is used (FxScale::ok, read by the host).
-__global__ void k_fx_scale(const unsigned long long* b, double Es, double Ep, int max_row, FxScale* out) {
+// dense: no product of the block is itself multiplied again, so coefficients may be twice as large;
+// four products a row and block limit rows to 32 blocks.
+__global__ void k_fx_scale(const unsigned long long* b, double Es, double Ep, int max_row, int dense, FxScale* out) {
     double v[4], lo[2];
     for (int m = 0; m < 4; ++m) v[m] = __longlong_as_double((long long)b[m]);
     for (int m = 0; m < 2; ++m) lo[m] = __longlong_as_double((long long)~b[4 + m]);
     FxScale s{};
-    s.ok = max_row <= 64;
+    s.ok = max_row <= (dense ? 32 : 64);
     for (int m = 0; m < 2; ++m)
         if (!(v[m] > 1e-100 && v[m] < 1e100 && v[m] <= 256.0 * lo[m] && v[2 + m] > 0.0)) s.ok = 0;
     if (s.ok) {
         const int row_bits = max_row <= 32 ? 61 : 59;
-        s.eH = min(56 - ilogb(v[2]), row_bits - ilogb(v[0]));
-        s.eS = min(56 - ilogb(v[3]), row_bits - ilogb(v[1]));
+        s.eH = min(56 + dense - ilogb(v[2]), row_bits - ilogb(v[0]));
+        s.eS = min(56 + dense - ilogb(v[3]), row_bits - ilogb(v[1]));
         s.Es = fx_split(fx_round(Es, s.eH));
         s.Ep = fx_split(fx_round(Ep, s.eH));
         s.one = fx_split(fx_round(1.0, s.eS));
@@ -106,11 +114,59 @@ __global__ void k_fx_records(int nnzb, const double* __restrict__ skr, const FxS
     rec[q] = fx_split(fx_round(skr[q], m < 4 ? 56 : m < 8 ? sc->eH : sc->eS));
 }
 
+// The same of caller matrices, dense 4 x 4 blocks: exact absolute row sums.
+__global__ void k_fx_bounds_dense(int n, const int* __restrict__ row_ptr, const double* __restrict__ H,
+                                  const double* __restrict__ S, unsigned long long* out) {
+    const int q = blockIdx.x * blockDim.x + threadIdx.x, i = q >> 2, r = q & 3;
+    unsigned long long w[6] = {0, 0, 0, 0, 0, 0};
+    if (i < n) {
+        for (int m = 0; m < 2; ++m) {
+            const double* X = m ? S : H;
+            double sum = 0.0, mx = 0.0;
+            for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e)
+                for (int c = 0; c < 4; ++c) {
+                    const double v = fabs(X[16 * (size_t)e + 4 * r + c]);
+                    sum += v;
+                    mx = fmax(mx, v);
+                }
+            if (!(sum <= 1e300)) sum = mx = 1e308;
+            w[m] = (unsigned long long)__double_as_longlong(sum);
+            w[2 + m] = (unsigned long long)__double_as_longlong(mx);
+            w[4 + m] = ~w[m];
+        }
+    }
+    for (int m = 0; m < 6; ++m) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long x = __shfl_xor_sync(0xffffffffu, w[m], o);
+            w[m] = x > w[m] ? x : w[m];
+        }
+        if ((threadIdx.x & 31) == 0) atomicMax(out + m, w[m]);
+    }
+}
+
+// Block records of caller matrices, 256 bytes each: H then S, row by row.
+__global__ void k_fx_records_dense(int nnzb, const double* __restrict__ H, const double* __restrict__ S,
+                                   const FxScale* __restrict__ sc, int2* __restrict__ rec) {
+    const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= 32 * (size_t)nnzb || !sc->ok) return;
+    const size_t e = q >> 5, m = q & 31;
+    rec[q] = m < 16 ? fx_split(fx_round(H[16 * e + m], sc->eH)) : fx_split(fx_round(S[16 * e + m - 16], sc->eS));
+}
+
+void fx_build_dense(int n, int nnzb, const int* row_ptr, const double* H, const double* S, int max_row,
+                    unsigned long long* bounds, FxScale* scale, int2* rec, cudaStream_t st) {
+    cudaMemsetAsync(bounds, 0, 6 * sizeof(unsigned long long), st);
+    k_fx_bounds_dense<<<(4 * n + 127) / 128, 128, 0, st>>>(n, row_ptr, H, S, bounds);
+    k_fx_scale<<<1, 1, 0, st>>>(bounds, 0.0, 0.0, max_row, 1, scale);
+    const size_t w = 32 * (size_t)nnzb;
+    k_fx_records_dense<<<(unsigned)((w + 255) / 256), 256, 0, st>>>(nnzb, H, S, scale, rec);
+}
+
 void fx_build(int n, int nnzb, const int* row_ptr, const int* col_idx, const double* skr, double Es, double Ep,
               int max_row, unsigned long long* bounds, FxScale* scale, int2* rec, cudaStream_t st) {
     cudaMemsetAsync(bounds, 0, 6 * sizeof(unsigned long long), st);
     k_fx_bounds<<<(n + 127) / 128, 128, 0, st>>>(n, row_ptr, col_idx, skr, Es, Ep, bounds);
-    k_fx_scale<<<1, 1, 0, st>>>(bounds, Es, Ep, max_row, scale);
+    k_fx_scale<<<1, 1, 0, st>>>(bounds, Es, Ep, max_row, 0, scale);
     const size_t w = 12 * (size_t)nnzb;
     k_fx_records<<<(unsigned)((w + 255) / 256), 256, 0, st>>>(nnzb, skr, scale, rec);
 }
@@ -208,7 +264,6 @@ struct FxState {
     int bH[NC], bS[NC];     // H u_n = f 2^bH P, S u_n = f 2^bS Y
     int sP[NC];             // lead: P = xd 2^sP, rounded
     double2* xd;            // lead: u_n (in units of X), then H u_n or w, in FP64
-    const double* skr;      // the FP64 block records
     double Es, Ep;
     double hh[2][NC];       // |P|^2 of the even and the odd steps
     int q[NC], done[NC], nue[NC], we[NC], big[NC];
@@ -322,7 +377,7 @@ struct FxTmem {
 };
 
 // The cluster of atom J: atoms, entries, and the rows of each group. Every thread of the CTA calls it.
-template <int NC, int T>
+template <int NC, int T, bool kDense>
 __device__ __forceinline__ void fx_view(const KrylovArgs& a, FxState<NC>& st, int J, int cbase, int n_at) {
     constexpr int G = T / NC;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -381,10 +436,10 @@ __device__ __forceinline__ void fx_view(const KrylovArgs& a, FxState<NC>& st, in
                 if (q >= n_at) break;
                 const bool in = ce[i] >= 0 && pos[i] >= 0 && cl[pos[i]] == ce[i];
                 if (q == qJ && in) at[r] = (short)pos[i];
-                const unsigned hit = __ballot_sync(0xffffffffu, in && pos[i] != q);
-                if (in && pos[i] != q)
+                const unsigned hit = __ballot_sync(0xffffffffu, in && (kDense || pos[i] != q));
+                if (in && (kDense || pos[i] != q))
                     ent[off[q] + cnt[i] + __popc(hit & ((1u << lane) - 1u))] =
-                        ((unsigned)fx_unit<NC>(pos[i], 0, 0) << 20) | (unsigned)(r * 96);
+                        ((unsigned)fx_unit<NC>(pos[i], 0, 0) << 20) | (unsigned)(r * (kDense ? 256 : 96));
                 cnt[i] += __popc(hit);
             }
         }
@@ -513,10 +568,76 @@ __device__ __forceinline__ void fx_products(FxState<NC>& st) {
     fx_or<NC>(mS, &st.bits[1][tc]);
 }
 
+// The same with dense 4 x 4 blocks, the on-site ones among the entries: 32 products an entry instead of
+// 16, 256 bytes of it instead of 96, which L2 has to deliver. H's block is applied while S's is on its
+// way, and S's while the next entry's H is. 512 atoms, nu 30, set_hs to density matrix: 27.9 ms with the
+// FP64 kernel, 11.7 ms (Slater-Koster form: 11.0 ms).
+template <int NC, int T>
+__device__ __forceinline__ void fx_products_dense(FxState<NC>& st) {
+    constexpr int G = T / NC;
+    const int tid = threadIdx.x, tc = tid % NC, g = tid / NC, NS = st.NS;
+    const short* row_at = fx_at<short>(st.v.row_at);
+    const char* const Xc = reinterpret_cast<const char*>(fx_at<int4>(st.v.X) + tc);
+    longlong2 *PH = fx_at<longlong2>(st.v.P), *PS = fx_at<longlong2>(st.v.Y);
+    unsigned long long mH = 0, mS = 0;
+#pragma unroll 1
+    for (int sl = 0; sl < NS; ++sl) {
+        const int q = row_at[sl * G + g];
+        if (q < 0) continue;
+        const unsigned* ent = fx_at<unsigned>(st.v.ent) + fx_at<int>(st.v.off)[q];
+        const char* rb = reinterpret_cast<const char*>(st.rec + 16 * (size_t)fx_at<int>(st.v.base)[q]);
+        const int d = fx_at<int>(st.v.deg)[q], u01 = fx_unit<NC>(q, 0, tc), u23 = fx_unit<NC>(q, 1, tc);
+        Fx H[4], S[4];
+        int4 hb[8], sb[8];
+        auto fetch = [&](unsigned en, int half, int4 (&b)[8]) {
+            const int4* at = reinterpret_cast<const int4*>(rb + (en & 0xffffu)) + 8 * half;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) b[i] = __ldg(at + i);
+        };
+        auto apply = [&](Fx (&y)[4], const int4 (&b)[8], const int4& x01, const int4& x23) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                fx_mac(y[r], fx_lo(b[2 * r]), fx_lo(x01));
+                fx_mac(y[r], fx_hi(b[2 * r]), fx_hi(x01));
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                fx_mac(y[r], fx_lo(b[2 * r + 1]), fx_lo(x23));
+                fx_mac(y[r], fx_hi(b[2 * r + 1]), fx_hi(x23));
+            }
+        };
+        unsigned en = d > 0 ? ent[0] : 0u;
+        if (d > 0) fetch(en, 0, hb);
+#pragma unroll 1
+        for (int k = 0; k < d; ++k) {
+            fetch(en, 1, sb);
+            const unsigned at = en >> 16;
+            const int4 x01 = *reinterpret_cast<const int4*>(Xc + at);
+            const int4 x23 = *reinterpret_cast<const int4*>(Xc + (at ^ (16u * NC)));
+            apply(H, hb, x01, x23);
+            en = ent[min(k + 1, d - 1)];
+            fetch(en, 0, hb);
+            apply(S, sb, x01, x23);
+        }
+        longlong2 y01 = make_longlong2(fx_fold(H[0]), fx_fold(H[1])), y23 = make_longlong2(fx_fold(H[2]), fx_fold(H[3]));
+        mH |= fx_abs_bits(y01.x) | fx_abs_bits(y01.y) | fx_abs_bits(y23.x) | fx_abs_bits(y23.y);
+        PH[u01] = y01;
+        PH[u23] = y23;
+        y01 = make_longlong2(fx_fold(S[0]), fx_fold(S[1]));
+        y23 = make_longlong2(fx_fold(S[2]), fx_fold(S[3]));
+        mS |= fx_abs_bits(y01.x) | fx_abs_bits(y01.y) | fx_abs_bits(y23.x) | fx_abs_bits(y23.y);
+        PS[u01] = y01;
+        PS[u23] = y23;
+    }
+    __syncwarp();
+    fx_or<NC>(mH, &st.bits[0][tc]);
+    fx_or<NC>(mS, &st.bits[1][tc]);
+}
+
 // The lead's form of fx_products: FP64 products of xd into P and Y (as FP64), entries whose neighbour
 // is not reached yet left out.
-template <int NC, int T>
-__device__ __forceinline__ void fx_products_lead(FxState<NC>& st) {
+template <int NC, int T, bool kDense>
+__device__ __forceinline__ void fx_products_lead(const KrylovArgs& a, FxState<NC>& st) {
     constexpr int G = T / NC;
     const int tid = threadIdx.x, tc = tid % NC, g = tid / NC, NS = st.NS;
     const short* row_at = fx_at<short>(st.v.row_at);
@@ -528,9 +649,14 @@ __device__ __forceinline__ void fx_products_lead(FxState<NC>& st) {
         const int q = row_at[sl * G + g];
         if (q < 0) continue;
         const unsigned* ent = fx_at<unsigned>(st.v.ent) + fx_at<int>(st.v.off)[q];
-        const char* rb = reinterpret_cast<const char*>(st.skr + 12 * (size_t)fx_at<int>(st.v.base)[q]);
+        const size_t b0 = (size_t)fx_at<int>(st.v.base)[q];
+        const char* rb = reinterpret_cast<const char*>(a.skr + 12 * b0);
         const int d = fx_at<int>(st.v.deg)[q], u01 = fx_unit<NC>(q, 0, tc), u23 = fx_unit<NC>(q, 1, tc);
-        double2 s01 = st.xd[u01], s23 = st.xd[u23];
+        double2 s01 = make_double2(0.0, 0.0), s23 = s01;
+        if (!kDense) {
+            s01 = st.xd[u01];
+            s23 = st.xd[u23];
+        }
         double2 h01 = make_double2(st.Es * s01.x, st.Ep * s01.y), h23 = make_double2(st.Ep * s23.x, st.Ep * s23.y);
 #pragma unroll 1
         for (int k = 0; k < d; ++k) {
@@ -538,6 +664,19 @@ __device__ __forceinline__ void fx_products_lead(FxState<NC>& st) {
             const double2 x01 = *reinterpret_cast<const double2*>(xc + at);
             const double2 x23 = *reinterpret_cast<const double2*>(xc + (at ^ (16u * NC)));
             if (x01.x == 0.0 && x01.y == 0.0 && x23.x == 0.0 && x23.y == 0.0) continue;
+            if (kDense) {
+                const size_t e = 16 * (b0 + (en & 0xffffu) / 256);
+                auto row = [&](const double* X, int r, double y) {
+                    const double2 c01 = __ldg(reinterpret_cast<const double2*>(X + e + 4 * r));
+                    const double2 c23 = __ldg(reinterpret_cast<const double2*>(X + e + 4 * r + 2));
+                    return fma(c23.y, x23.y, fma(c23.x, x23.x, fma(c01.y, x01.y, fma(c01.x, x01.x, y))));
+                };
+                h01 = make_double2(row(a.H, 0, h01.x), row(a.H, 1, h01.y));
+                h23 = make_double2(row(a.H, 2, h23.x), row(a.H, 3, h23.y));
+                s01 = make_double2(row(a.S, 0, s01.x), row(a.S, 1, s01.y));
+                s23 = make_double2(row(a.S, 2, s23.x), row(a.S, 3, s23.y));
+                continue;
+            }
             const double2* r = reinterpret_cast<const double2*>(rb + (en & 0xffffu));
             const double2 u = __ldg(r), uz = __ldg(r + 1), a01 = __ldg(r + 2), a23 = __ldg(r + 3);
             const double2 b01 = __ldg(r + 4), b23 = __ldg(r + 5);
@@ -719,13 +858,13 @@ __device__ __forceinline__ void fx_pass_a(FxState<NC>& st, int n) {
 // the integers' products; u_n = f X, S u_n = f 2^bS Y, H u_n = f 2^bH P.
 //
 // X^T S X, and whether u_n exists: the tests on w = 2^we X times the scale of H u_(n-1) (n > 0)
-// against its norm, w^T S w against that of H u_(n-1), both without the common scale. Returns 0, or
-// 1 (no new direction) or 2 (S not positive definite).
+// against its norm, w^T S w against that of H u_(n-1), both without the common scale. Returns 0, 1
+// (no new direction), 2 (S not positive definite) or 3 (S_jj <= 0).
 template <int NC>
 __device__ __forceinline__ int fx_norm_test(const KrylovArgs& a, const FxState<NC>& st, int n, int c, double& xsx) {
     const int nm = st.nm, RC = 3 * nm + 1;
     xsx = fx_red_get(fx_at<int>(st.v.red) + c * RC + nm + n, NC * RC) * fx_pow2(60 + st.bS[c]);
-    if (n == 0) return 0;
+    if (n == 0) return xsx > 0.0 ? 0 : 3;
     const double w2 = xsx * fx_pow2(2 * st.we[c]), bound = a.breakdown_tol * a.breakdown_tol * st.hh[(n - 1) & 1][c];
     return w2 < -bound ? 2 : w2 > bound ? 0 : 1;
 }
@@ -744,7 +883,7 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
     const int stop = fx_norm_test(a, st, n, c, xsx);
     if (stop) {
         if (lane == 0) {
-            if (stop == 2) flag(a.status, DEV_NOT_SPD);
+            if (stop > 1) flag(a.status, stop == 2 ? DEV_NOT_SPD : DEV_ARG);
             st.nue[c] = n;
             st.done[c] = 1;
             atomicSub(&st.live, 1);
@@ -1160,9 +1299,11 @@ __device__ __forceinline__ void fx_results(const KrylovArgs& a, FxState<NC>& st,
     __syncthreads();
 }
 
-template <int NC, int T, int kMinB>
+// kDense: caller matrices (dense blocks) instead of two-centre ones.
+template <int NC, int T, int kMinB, bool kDense>
 __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant__ KrylovArgs a, const __grid_constant__ FxArgs x) {
     __shared__ FxState<NC> st;
+    if (!x.scale->ok) return;   // (caller matrices: the FP64 kernel takes them)
     using Tm = FxTmem<T, kMinB>;
     if (threadIdx.x == 0) {
         const size_t cta_units = (size_t)a.nu_max * a.na_max * 2 * NC;
@@ -1172,7 +1313,6 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
         st.gU = reinterpret_cast<int4*>(a.scratch) + (2 * cta_units + (size_t)a.na_max * 2 * NC) * blockIdx.x;
         st.gY = st.gU + cta_units;
         st.gX = st.gY + cta_units;
-        st.skr = a.skr;
         st.Es = x.Es;
         st.Ep = x.Ep;
         st.nm = a.nu_max;
@@ -1214,7 +1354,7 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
             __syncthreads();
             continue;
         }
-        fx_view<NC, T>(a, st, J, a.cl_ptr ? a.cl_ptr[J] : 0, st.n_at);
+        fx_view<NC, T, kDense>(a, st, J, a.cl_ptr ? a.cl_ptr[J] : 0, st.n_at);
         if (a.bstore)
             balanced_positions<32, T>(st.n_at, (st.n_at + 31) / 32, fx_at<int>(st.v.deg), fx_at<int>(st.v.pos),
                                       fx_at<int>(st.v.pos_atom));
@@ -1222,7 +1362,8 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
             fx_start<NC, T, kMinB>(st);
             const int nu = st.nu;
             for (int n = 0; n < nu; ++n) {
-                if (n < kLead) fx_products_lead<NC, T>(st);
+                if (n < kLead) fx_products_lead<NC, T, kDense>(a, st);
+                else if constexpr (kDense) fx_products_dense<NC, T>(st);
                 else fx_products<NC, T>(st);
                 __syncthreads();
                 fx_take_products<NC, T>(st, n);
@@ -1279,11 +1420,12 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
 namespace {
 struct FxForm {
     int nc, t, min_b;       // columns at a time, threads, CTAs an SM holds
-    const void* fn;
+    const void *fn, *fn_dense;
     FxLayout (*layout)(int, int, int, bool, bool);
 };
 template <int NC, int T, int B>
-FxForm fx_form() { return {NC, T, B, reinterpret_cast<const void*>(&k_krylov_fixed<NC, T, B>), &fx_layout<NC, T>}; }
+FxForm fx_form() { return {NC, T, B, reinterpret_cast<const void*>(&k_krylov_fixed<NC, T, B, false>),
+            reinterpret_cast<const void*>(&k_krylov_fixed<NC, T, B, true>), &fx_layout<NC, T>}; }
 const FxForm kForms[] = {fx_form<4, 384, 1>(), fx_form<1, 128, 2>()};
 constexpr int kMaxUpt = 7;      // units of a thread: eight lanes' sums of 2 x 7 products of 2^112 / 2^56 stay below 2^63
 constexpr size_t kSmemSM = 233472, kSmemCta = 232448;   // per SM, and the most one CTA may have
@@ -1326,13 +1468,14 @@ void fx_columns(const KrylovArgs& a, FxArgs x, int form, int grid, int ctas_per_
     const size_t share = std::min(kSmemCta, kSmemSM / ctas_per_sm - 1024) - kSmemStatic;
     x.smem_bytes = (int)(std::min(all, share) & ~(size_t)15);
     x.split = f.nc < 4;
+    const void* fn = a.skr ? f.fn : f.fn_dense;
     cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, f.fn) != cudaSuccess || fa.maxDynamicSharedSizeBytes < x.smem_bytes) {
-        cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, x.smem_bytes);
-        cudaFuncSetAttribute(f.fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess || fa.maxDynamicSharedSizeBytes < x.smem_bytes) {
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, x.smem_bytes);
+        cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     }
     void* args[] = {const_cast<KrylovArgs*>(&a), &x};
-    cudaLaunchKernel(f.fn, dim3(grid), dim3(f.t), args, (size_t)x.smem_bytes, st);
+    cudaLaunchKernel(fn, dim3(grid), dim3(f.t), args, (size_t)x.smem_bytes, st);
 }
 
 }  // namespace elses

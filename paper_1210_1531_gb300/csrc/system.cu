@@ -132,7 +132,7 @@ int prepare_columns(elses_system s) {
     };
     for (int b = 0; b < s->n; b += s->batch_atoms) {
         const int e = std::min(s->n, b + s->batch_atoms);
-        size_t batch_off = 0, fp64_off = 0;
+        size_t batch_off = 0;
         for (int ns = s->na_max / gslot; ns >= 1; --ns) {
             const int key = gslot * ns / 16;
             const bool half = half_ok && (ns & 1) && odd_half(key);
@@ -156,25 +156,29 @@ int prepare_columns(elses_system s) {
             if (bps < 1) return fail(ELSES_ERR_CAPACITY, "Krylov kernel cannot be resident (%d-atom class)", na);
             // a count fixed by the caller or chosen by the autotuner may use the 4-CTA form
             int bps_max = (s->p.krylov_block || half) ? bps : krylov_blocks_per_sm_max(na, kdeg);
-            int fx = -1;
-            // scratch for the FP64 kernels too: elses_set_hs returns to them without a reallocation
-            fp64_off += (size_t)std::min(count, s->num_sms * bps) * kWarpsPerAtom * 2 * nm * na * 4;
-            if (fx_ok) {
-                const int form = fx_form_for(s->n, s->num_sms);
-                const int nb = fx_blocks_per_sm(form, na, s->max_nb, nm, s->p.reorth != 0, s->p.force_mode == 1);
-                if (nb > 0) {
-                    fx = form;
-                    bps = bps_max = nb;
-                }
+            int fx = -1, fx_dense = -1;
+            const int form = fx_form_for(s->n, s->num_sms);
+            const int fx_b = s->p.krylov_block ? 0 : fx_blocks_per_sm(form, na, s->max_nb + 1, nm, s->p.reorth != 0, s->p.force_mode == 1);
+            const auto shape = [&](bool fixed, int b, int b_max) {
+                if (s->p.k3_ctas_per_sm > 0) return std::min(b_max, s->p.k3_ctas_per_sm);
+                if (key < (int)s->tuned_bps.size() && s->tuned_bps[key] > 0 && s->tuned_fx[key] == fixed)
+                    return std::min(b_max, s->tuned_bps[key]);
+                return b;
+            };
+            bps = shape(false, bps, bps_max);
+            const int bps64 = bps, grid64 = std::min(count, s->num_sms * bps);
+            if (fx_b > 0) {
+                fx_dense = form;
+                if (fx_ok) fx = form;
             }
-            if (s->p.k3_ctas_per_sm > 0) bps = std::min(bps_max, s->p.k3_ctas_per_sm);
-            else if (key < (int)s->tuned_bps.size() && s->tuned_bps[key] > 0) bps = std::min(bps_max, s->tuned_bps[key]);
+            if (fx >= 0) bps = shape(true, fx_b, fx_b);
             const int grid = std::min(fx >= 0 ? fx_items(fx, count) : count, s->num_sms * bps);
-            s->k3_launches.push_back({b, e, begin, count, na, grid, bps, half ? 1 : 0, key, fx, batch_off});
-            batch_off += s->p.krylov_block ? (size_t)grid * block_krylov_scratch_doubles(nm, na)
-                         : fx >= 0         ? (size_t)grid * fx_scratch_doubles(fx, nm, na)
-                                           : (size_t)grid * kWarpsPerAtom * 2 * nm * na * 4;
-            scratch = std::max(scratch, fx_ok ? std::max(batch_off, fp64_off) : batch_off);
+            s->k3_launches.push_back({b, e, begin, count, na, grid, bps, half ? 1 : 0, key, fx, fx_dense, grid64, bps64, batch_off});
+            // scratch for the kernel with the largest need, as caller matrices change it without a new plan
+            const size_t fp64 = (size_t)grid64 * kWarpsPerAtom * 2 * nm * na * 4;
+            const size_t fixed = fx_dense >= 0 ? (size_t)std::min(fx_items(form, count), s->num_sms * fx_b) * fx_scratch_doubles(form, nm, na) : 0;
+            batch_off += s->p.krylov_block ? (size_t)grid * block_krylov_scratch_doubles(nm, na) : std::max(fp64, fixed);
+            scratch = std::max(scratch, batch_off);
             if (count > best_items) { best_items = count; s->k3_bps = bps; }
         }
     }
@@ -498,7 +502,17 @@ int run_batch(elses_system s, int b, int e, bool stored, double** V_out, int* v_
             CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int), lst));
             ka.queue = q;
         }
-        launch_krylov(s, ka, L.fx, L.grid, L.bps, lst);
+        if (s->user_hs && s->fx_user && L.fx_dense >= 0) {
+            // the fixed-point kernel where the matrices suit it, decided on the device, else the FP64 one
+            const int fb = fx_blocks_per_sm(L.fx_dense, L.na, s->max_nb + 1, s->nu_max, s->p.reorth != 0, s->p.force_mode == 1);
+            const int bps = s->p.k3_ctas_per_sm > 0 ? std::min(fb, s->p.k3_ctas_per_sm) : fb;
+            launch_krylov(s, ka, L.fx_dense, std::min(fx_items(L.fx_dense, L.item_count), s->num_sms * bps), bps, lst);
+            s->stats.launches++;
+            ka.skip = &s->fx_scale.p->ok;
+        }
+        if (s->user_hs) launch_krylov(s, ka, -1, L.grid64, L.bps64, lst);
+        else launch_krylov(s, ka, L.fx, L.grid, L.bps, lst);
+        ka.skip = nullptr;
         s->stats.launches++;
         s->stats.krylov_launches++;
     }
@@ -1089,13 +1103,18 @@ int elses_set_hs(elses_system s, int nnzb, const int* row_ptr_dev, const int* co
         s->drop_graph();
         TRY(prepare_columns(s));
     }
-    if (!s->user_hs && s->fx) {   // the launch plan of the FP64 kernels
-        s->user_hs = true;
-        TRY(prepare_columns(s));
-    }
     s->user_hs = true;
     CUDA_TRY(cudaMemcpyAsync(s->H.p, H_dev, sizeof(double) * 16 * s->nnzb, cudaMemcpyDeviceToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(s->S.p, S_dev, sizeof(double) * 16 * s->nnzb, cudaMemcpyDeviceToDevice, st));
+    // records for the fixed-point kernel (their buffer is not allocated while the stream is captured)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+    s->fx_user = !s->p.krylov_block && (cap == cudaStreamCaptureStatusNone || s->fx_rec.cap >= 32 * (size_t)s->nnzb);
+    if (s->fx_user) {
+        TRY(s->fx_rec.ensure(32 * (size_t)s->nnzb));
+        fx_build_dense(s->n, s->nnzb, s->row_ptr.p, s->H.p, s->S.p, s->max_nb, s->fx_bounds.p, s->fx_scale.p, s->fx_rec.p, st);
+        s->stats.launches += 3;
+    }
     s->have_rho = false;
     s->v_lazy = false;   // every column is recomputed before V is used again
     s->v_arch = false;

@@ -100,6 +100,7 @@ struct elses_system_s {
 
     int nu_max = 0, na_max = 0, k3_grid = 0, batch_atoms = 0, deg_cap = 0, k3_bps = 0;
     std::vector<int> tuned_bps;            // autotuner: resident Krylov CTAs per SM by class capacity / 16
+    std::vector<char> tuned_fx;            // whether that was the fixed-point kernel
     std::vector<int> tuned_order;          // autotuner: work-queue order by class capacity / 16 (1 size, 2 atom)
     std::vector<int> tuned_half;           // autotuner: odd 16-slot classes, 1 half-warps, 2 whole warps
     // Krylov launches: per batch of atoms, one launch per cluster size class (slots of 32 atoms),
@@ -108,8 +109,13 @@ struct elses_system_s {
     // batch can run at the same time
     // key: the class's bound on cluster size in slots of 16 atoms (its capacity na may be larger)
     // fx: the form of the fixed-point kernel that runs the class, -1 the FP64 kernels
-    struct K3Launch { int batch_begin, batch_end, item_begin, item_count, na, grid, bps, half, key, fx; size_t scratch_off; };
+    // and fx_dense with caller matrices; grid64, bps64: the FP64 kernels' shape
+    struct K3Launch {
+        int batch_begin, batch_end, item_begin, item_count, na, grid, bps, half, key, fx, fx_dense, grid64, bps64;
+        size_t scratch_off;
+    };
     bool fx = false;                       // the fixed-point Krylov form suits the system's H and S
+    bool fx_user = false;                  // caller matrices have records (fx_scale->ok says whether they are used)
     DevBuf<elses::FxScale> fx_scale;
     DevBuf<unsigned long long> fx_bounds;
     DevBuf<int2> fx_rec;

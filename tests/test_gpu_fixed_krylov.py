@@ -1,5 +1,7 @@
-"""The fixed-point Krylov kernel (Slater-Koster systems) against the FP64 one, which the same H and S
-take when the caller sets them (elses_set_hs), at the sizes where the former's work is split: the
+"""The fixed-point Krylov kernel, of Slater-Koster systems and of a caller's matrices (elses_set_hs),
+against the FP64 one, which takes over where the rows of H or S differ too much in size: the basis
+functions of an atom on its own are scaled by 32, which is exact and changes nothing but that atom's
+block of rho. At the sizes where the work is split: the
 units of a thread (128 and 384 threads), vectors in tensor memory, shared memory and scratch, the
 first steps in FP64, clusters it leaves to the FP64 kernel, both Gram-Schmidt forms, kept bases.
 
@@ -29,16 +31,27 @@ def _system(n, seed=3):
     return np.ascontiguousarray(pos[:n]), box
 
 
-def _pair(eg, pos, box, r_cluster, nu, **kw):
+def _forms(eg, n, r_cluster, nu, **kw):
+    """The system of n atoms (the last on its own in a vacuum), the same as caller matrices, the same
+    with the last atom's functions scaled, and that scale by block of H, S and rho."""
+    pos, box = _system(n - 1)
+    box = np.array(box, dtype=np.float64)
+    pos = np.concatenate([pos, [[0.0, 0.0, box[2] + 10.0]]])
+    box[2] += 20.0
     make = lambda: eg.System(torch.tensor(pos, device="cuda"), box, wl.sk_params(), r_cluster, nu, 0.1,  # noqa: E731
-                             4.0 * len(pos), **kw)
-    a, b = make(), make()
-    b.set_hs(*a.hs())
-    return a, b
+                             4.0 * n, **kw)
+    sk, caller, fp64 = make(), make(), make()
+    H, S = sk.hs()
+    caller.set_hs(H, S)
+    d = torch.ones_like(H)
+    d[-1] = 1024.0
+    assert int(sk.pattern()[0][-2]) == len(H) - 1
+    fp64.set_hs(H * d, S * d)
+    return sk, caller, fp64, d
 
 
 @pytest.mark.parametrize("n, nu, r_cluster, reorth", [
-    (1, 3, 0.0, 0), (2, 8, 0.0, 1),                                  # a single atom, a pair
+    (2, 3, 0.0, 0), (3, 8, 0.0, 1),                                  # single atoms, a pair
     (63, 1, 0.0, 0), (64, 2, 0.0, 1), (65, 3, 0.0, 0),               # one column per CTA: 126, 128, 130 units
     (64, 4, 0.0, 0), (65, 5, 0.0, 1), (64, 33, 0.0, 0),              # around the FP64 steps; past a warp of vectors
     (72, 64, 0.0, 1),                                                # the largest nu
@@ -46,17 +59,42 @@ def _pair(eg, pos, box, r_cluster, nu, **kw):
     (512, 21, 4.3, 0), (512, 30, 6.0, 1), (500, 30, 5.1, 0),         # four columns per CTA, ragged clusters
 ])
 def test_matches_the_fp64_kernel(eg, n, nu, r_cluster, reorth):
-    pos, box = _system(n)
-    a, b = _pair(eg, pos, box, r_cluster, nu, reorth=reorth)
-    a.green_columns()
-    b.green_columns()
-    mu, _ = a.find_mu()
-    sa, sb = a.spectra(), b.spectra()
-    assert torch.equal(sa["nu_eff"], sb["nu_eff"])
-    for x, y in zip(a.density_matrix(mu), b.density_matrix(mu)):
-        assert float((x - y).abs().max()) <= RHO_TOL * float(y.abs().max())
-    ea, eb = a.energies(mu), b.energies(mu)
-    assert abs(ea["E_band"] - eb["E_band"]) <= 1e-12 * abs(eb["E_band"])
+    sk, caller, fp64, d = _forms(eg, n, r_cluster, nu, reorth=reorth)
+    for s in (sk, caller, fp64):
+        s.green_columns()
+    mu, _ = fp64.find_mu()
+    ref = [x * d for x in fp64.density_matrix(mu)]
+    e_ref, sp_ref = fp64.energies(mu)["E_band"], fp64.spectra()
+    for s in (sk, caller):
+        assert torch.equal(s.spectra()["nu_eff"], sp_ref["nu_eff"])
+        for x, y in zip(s.density_matrix(mu), ref):
+            assert float((x - y).abs().max()) <= RHO_TOL * float(y.abs().max())
+        assert abs(s.energies(mu)["E_band"] - e_ref) <= 1e-12 * abs(e_ref)
+
+
+def test_caller_matrices_under_capture_and_after_other_matrices(eg):
+    """The choice of kernel is made on the device with every set_hs, also in a captured one."""
+    sk, caller, fp64, d = _forms(eg, 64, 0.0, 12)
+    H, S = sk.hs()
+    caller.green_columns()
+    fp64.green_columns()
+    want, want64 = caller.spectra()["eps"].clone(), fp64.spectra()["eps"].clone()
+    Hin, Sin = H.clone(), S.clone()
+    st = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(st):
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=st):
+            caller.set_hs(Hin, Sin, stream=st)
+    for f, w in ((1.0, want), (d, want64), (1.0, want)):
+        Hin.copy_(H * f)
+        Sin.copy_(S * f)
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        caller.set_hs(Hin, Sin)
+        caller.green_columns()
+        assert torch.equal(caller.spectra()["eps"], w)
 
 
 def test_results_do_not_depend_on_batches_or_schedule(eg):
