@@ -13,7 +13,12 @@
 //                  (lanes over rows / columns); the three vectors z = L^-1 (U, SU, HU)_j are
 //                  reflected along, y = Q_H^T z.
 //   k_eig_chase    one thread per column: implicit-shift QR sweeps on T (Wilkinson shift, Givens
-//                  bulge chase) -- the sequential part; the rotations are recorded.
+//                  bulge chase) -- the sequential part; the rotations are recorded. A warp issues one
+//                  FP64 instruction in 64 clocks and there is less than one warp per scheduler up to
+//                  19456 columns, so the time is their number: the update by way of p = s t (Bowdler,
+//                  Martin, Reinsch and Wilkinson's form) instead of D and E each from c^2, s^2 and
+//                  c s, and tests for small entries on the exponents as integers, take 20 a rotation
+//                  instead of 32: 1.72 -> 1.20 ms (256 columns, nu 30), 1.85 -> 1.32 ms (16384).
 //   k_eig_spectra  one thread per (column, vector): the rotations replayed on y give
 //                  c, d, g = Q^T z.
 //   k_eig_vectors  one warp per column, only where V itself is needed (G(z), the adjoint, or
@@ -275,7 +280,12 @@ __global__ void __launch_bounds__(kChaseThreads) k_eig_chase(const EigArgs a) {
     const size_t cap = eig_rot_cap(nm);
     size_t nrot = 0;
     bool ok = true;
-    const double eps = 2.220446049250313e-16;
+    // |E_k| <= 2^-52 max(|D_k|, |D_k+1|), to the last of the 20 mantissa bits of their upper words
+    auto negligible = [&](int k) {
+        const int e = __double2hiint(E[k]) & 0x7fffffff;
+        const int d = max(__double2hiint(D[k]) & 0x7fffffff, __double2hiint(D[k + 1]) & 0x7fffffff);
+        return e == 0 || e + (52 << 20) <= d;
+    };
     int hi = nu - 1, sweeps = 0;
     const int max_sweeps = a.max_sweeps > 0 ? a.max_sweeps : 30 * nu;
     // each pass deflates every negligible trailing off-diagonal entry, then makes one sweep:
@@ -283,13 +293,13 @@ __global__ void __launch_bounds__(kChaseThreads) k_eig_chase(const EigArgs a) {
     // otherwise sit out the other lanes' sweep), in the same order of operations per column.
     // A column without a space (nu = 0, flagged by the Krylov build) has nothing to chase.
     while (ok && hi > 0) {
-        while (hi > 0 && fabs(E[hi - 1]) <= eps * (fabs(D[hi - 1]) + fabs(D[hi]))) {
+        while (hi > 0 && negligible(hi - 1)) {
             E[hi - 1] = 0.0;
             --hi;
         }
         if (hi == 0) break;
         int lo = hi - 1;
-        while (lo > 0 && fabs(E[lo - 1]) > eps * (fabs(D[lo - 1]) + fabs(D[lo]))) --lo;
+        while (lo > 0 && !negligible(lo - 1)) --lo;
         if (lo > 0) E[lo - 1] = 0.0;
         if (++sweeps > max_sweeps || nrot + (hi - lo) > cap) {
             ok = false;
@@ -299,34 +309,37 @@ __global__ void __launch_bounds__(kChaseThreads) k_eig_chase(const EigArgs a) {
         const double b2 = E[hi - 1] * E[hi - 1];
         const double den = delta + copysign(sqrt(delta * delta + b2), delta);
         const double mu = D[hi] - (den != 0.0 ? b2 / den : 0.0);
-        double x = D[lo] - mu, z = E[lo];
+        // The rotation of k, k + 1: x the entry to keep, s e the one to remove, g = D_k, b = E_k after the
+        // rotation before, t = s (D_k+1 - g) + 2 c b; D_k = g + s t, D_k+1 -= s t, E_k = c t - b.
+        double x = D[lo] - mu, cr = 1.0, sr = 1.0, p = 0.0;
         for (int k = lo; k < hi; ++k) {
+            const double e = E[k], z = sr * e, b = cr * e;
             // c = x / r, s = z / r, r = |(x, z)| from one reciprocal square root
             const double rr = fma(x, x, z * z);
-            double cr = 1.0, sr = 0.0, r = 0.0;
-            if (rr > 0.0) {
+            double r = 0.0;
+            cr = 1.0;
+            sr = 0.0;
+            if (__double2hiint(rr) > 0) {
                 const double ir = rsqrt(rr);
                 cr = x * ir;
                 sr = z * ir;
                 r = rr * ir;
             }
             if (k > lo) E[k - 1] = r;
-            const double ak = D[k], ak1 = D[k + 1], b = E[k];
-            const double cc = cr * cr, ss = sr * sr, cs = cr * sr;
-            D[k] = cc * ak + 2.0 * cs * b + ss * ak1;
-            D[k + 1] = ss * ak - 2.0 * cs * b + cc * ak1;
-            E[k] = cs * (ak1 - ak) + (cc - ss) * b;
-            if (k + 1 < hi) {
-                const double bn = E[k + 1];
-                z = sr * bn;
-                E[k + 1] = cr * bn;
-                x = E[k];
-            }
+            const double g = D[k] - p;
+            // 2 c by its exponent (c = 0 becomes 2^-1022)
+            const double c2 = __hiloint2double(__double2hiint(cr) + (1 << 20), __double2loint(cr));
+            const double t = fma(D[k + 1] - g, sr, c2 * b);
+            p = sr * t;
+            D[k] = g + p;
+            x = fma(cr, t, -b);
             rc[nrot] = cr;
             rs[nrot] = sr;
             rk[nrot] = (unsigned char)k;
             ++nrot;
         }
+        D[hi] -= p;
+        E[hi - 1] = x;
     }
     if (!ok) flag(a.status, DEV_TIMEOUT);
     a.rot_n[c] = ok ? (int)nrot : 0;
