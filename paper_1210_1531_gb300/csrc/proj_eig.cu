@@ -8,8 +8,8 @@
 //
 // GB300 form. On this part the FP64 pipe charges a whole warp instruction whatever the number
 // of active lanes, so every FP64 instruction must carry work on all lanes:
-//   k_eig_reduce   one warp per column, matrices in shared memory: Cholesky, the reduction
-//                  A = L^-1 H' L^-T and the Householder reduction of A to tridiagonal form T
+//   k_eig_reduce   one warp per column, matrices in shared memory: Cholesky (or, where S' = I to
+//                  2^-32, its first-order form), the reduction A = L^-1 H' L^-T and the Householder reduction of A to tridiagonal form T
 //                  (lanes over rows / columns); the three vectors z = L^-1 (U, SU, HU)_j are
 //                  reflected along, y = Q_H^T z.
 //   k_eig_chase    one thread per column: implicit-shift QR sweeps on T (Wilkinson shift, Givens
@@ -71,29 +71,10 @@ __device__ __forceinline__ double packed(const double* P, int i, int k) {
 }
 
 // ----------------------------------------------------------------------------- k_eig_reduce
-__global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
-    extern __shared__ __align__(16) double sm[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int c = blockIdx.x * (blockDim.x >> 5) + wib;
-    if (c >= a.ncols) return;
-    const int nm = a.nu_max, ld = nm + 1;
-    double* A = sm + (size_t)wib * ((2 * nm + 3) * ld + 2 * nm + 3);
-    double* L = A + (nm + 3) * ld;  // A: the matrix, then the three vectors as rows nu .. nu + 2
-    double* inv = L + nm * ld;     // 1 / L_ii
-    double* P = inv + nm;          // Householder work vector (nm + 3)
-    double* yv = a.tri + (size_t)c * eig_tri_doubles(nm);   // D, E, yc, yd, yg (global)
-    const int j = a.col0 + c;
-    const int nu = a.nu_eff[j];
-    const int PK = nm * (nm + 1) / 2;
-    const double* Hp = a.Hp + (size_t)c * PK;
-    const double* Sp = a.Sp + (size_t)c * PK;
-
-    for (int q = lane; q < nu * nu; q += 32) {
-        const int i = q / nu, k = q % nu;
-        A[i * ld + k] = packed(Hp, i, k);
-        L[i * ld + k] = packed(Sp, i, k);
-    }
-    __syncwarp();
+// S' = L L^T, A = L^-1 H' L^-T and z = L^-1 (U, SU, HU)_j into rows nu .. nu + 2 of A, in the general
+// form; false where S' is not positive definite.
+__device__ __forceinline__ bool reduce_cholesky(double* A, double* L, double* inv, int nu, int ld, int lane,
+                                                const double* z_u, const double* z_s, const double* z_h) {
     // Cholesky S' = L L^T (right-looking, lanes over rows of the trailing block)
     bool spd = true;
     for (int k = 0; k < nu; ++k) {
@@ -109,11 +90,7 @@ __global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
         });
         __syncwarp();
     }
-    if (!spd) {
-        if (lane == 0) flag(a.status, DEV_NOT_SPD);
-        for (int q = lane; q < 5 * nm; q += 32) yv[q] = 0.0;
-        return;
-    }
+    if (!spd) return false;
     // X = L^-1 H' in place (lanes over columns n), then A = X L^-T in place (lanes over rows i)
     for (int n = lane; n < nu; n += 32)
         for (int i = 0; i < nu; ++i) {
@@ -139,7 +116,7 @@ __global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
     // the three vectors z = L^-1 (U, SU, HU)_j into rows nu .. nu + 2 of A: a column sweep with
     // lanes over rows (rows lane and lane + 32), row m final at step m
     {
-        const double* src[3] = {a.urow + (size_t)c * nm, a.surow + (size_t)c * nm, a.hurow + (size_t)c * nm};
+        const double* src[3] = {z_u, z_s, z_h};
         double z0[3], z1[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -176,6 +153,98 @@ __global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
             if (lane + 32 < nu) A[(nu + q) * ld + lane + 32] = z1[q];
         }
     }
+    return true;
+}
+
+// The same for S' = I + E with |E| < 2^-32, as Gram-Schmidt leaves it: L = I + T with T the strict lower
+// triangle of E and half its diagonal, L^-1 = I - T, up to products of E that are below 2^-64. What T
+// changes in H' and z is below 2^-32 of them, so FP32 sums carry it to 2^-56, without an FP64
+// instruction: the kernel at 16384 columns and nu 30 takes 3.29 ms in the general form and 2.05 ms in
+// this one (0.1 ms of it from the Householder norm by one reciprocal square root). Nothing reads the
+// upper triangles after this: they hold T and H' in FP32 meanwhile.
+__device__ __forceinline__ void reduce_unit(double* A, double* L, double* P, int nu, int ld, int lane,
+                                            const double* z_u, const double* z_s, const double* z_h) {
+    auto f32 = [](double* X, int at) -> float& { return *reinterpret_cast<float*>(X + at); };
+    float2* const diag = reinterpret_cast<float2*>(P);   // T_ii, H'_ii
+    lower_pairs(0, nu, lane, [&](int i, int m) {
+        const double e = L[i * ld + m], h = A[i * ld + m];
+        if (i == m) {
+            const double t = 0.5 * (e - 1.0);
+            L[i * ld + i] = 1.0 + t;
+            diag[i] = make_float2((float)t, (float)h);
+        } else {
+            f32(L, m * ld + i) = (float)e;
+            f32(A, m * ld + i) = (float)h;
+        }
+    });
+    __syncwarp();
+    lower_pairs(0, nu, lane, [&](int i, int k) {   // (T H' + H' T^T)_ik
+        float s0 = 0.0f, s1 = 0.0f;
+        for (int m = 0; m < k; ++m) {
+            s0 = fmaf(f32(L, m * ld + i), f32(A, m * ld + k), s0);
+            s1 = fmaf(f32(L, m * ld + k), f32(A, m * ld + i), s1);
+        }
+        if (i == k) {
+            s0 = fmaf(2.0f * diag[i].x, diag[i].y, s0);
+        } else {
+            const float hik = f32(A, k * ld + i);
+            s0 = fmaf(f32(L, k * ld + i), diag[k].y, s0);
+            s1 = fmaf(diag[k].x + diag[i].x, hik, s1);
+            for (int m = k + 1; m < i; ++m) s0 = fmaf(f32(L, m * ld + i), f32(A, k * ld + m), s0);
+        }
+        A[i * ld + k] -= (double)(s0 + s1);
+    });
+    const double* src[3] = {z_u, z_s, z_h};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double z0 = lane < nu ? src[q][lane] : 0.0, z1 = lane + 32 < nu ? src[q][lane + 32] : 0.0;
+        const float f0 = (float)z0, f1 = (float)z1;
+        float s0 = 0.0f, s1 = 0.0f;
+        for (int m = 0; m < nu; ++m) {
+            const float zm = __shfl_sync(0xffffffffu, m < 32 ? f0 : f1, m & 31);
+            if (lane >= m && lane < nu) s0 = fmaf(lane == m ? diag[m].x : f32(L, m * ld + lane), zm, s0);
+            if (lane + 32 >= m && lane + 32 < nu) s1 = fmaf(lane + 32 == m ? diag[m].x : f32(L, m * ld + lane + 32), zm, s1);
+        }
+        if (lane < nu) A[(nu + q) * ld + lane] = z0 - (double)s0;
+        if (lane + 32 < nu) A[(nu + q) * ld + lane + 32] = z1 - (double)s1;
+    }
+}
+
+__global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
+    extern __shared__ __align__(16) double sm[];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int c = blockIdx.x * (blockDim.x >> 5) + wib;
+    if (c >= a.ncols) return;
+    const int nm = a.nu_max, ld = nm + 1;
+    double* A = sm + (size_t)wib * ((2 * nm + 3) * ld + 2 * nm + 3);
+    double* L = A + (nm + 3) * ld;  // A: the matrix, then the three vectors as rows nu .. nu + 2
+    double* inv = L + nm * ld;     // 1 / L_ii
+    double* P = inv + nm;          // Householder work vector (nm + 3)
+    double* yv = a.tri + (size_t)c * eig_tri_doubles(nm);   // D, E, yc, yd, yg (global)
+    const int j = a.col0 + c;
+    const int nu = a.nu_eff[j];
+    const int PK = nm * (nm + 1) / 2;
+    const double* Hp = a.Hp + (size_t)c * PK;
+    const double* Sp = a.Sp + (size_t)c * PK;
+
+    bool unit = true;      // S' = I to 2^-32
+    for (int q = lane; q < nu * nu; q += 32) {
+        const int i = q / nu, k = q % nu;
+        const double s = packed(Sp, i, k);
+        A[i * ld + k] = packed(Hp, i, k);
+        L[i * ld + k] = s;
+        unit = unit && fabs(i == k ? s - 1.0 : s) < 0x1p-32;
+    }
+    unit = __all_sync(0xffffffffu, unit);
+    __syncwarp();
+    if (unit) {
+        reduce_unit(A, L, P, nu, ld, lane, a.urow + (size_t)c * nm, a.surow + (size_t)c * nm, a.hurow + (size_t)c * nm);
+    } else if (!reduce_cholesky(A, L, inv, nu, ld, lane, a.urow + (size_t)c * nm, a.surow + (size_t)c * nm,
+                                a.hurow + (size_t)c * nm)) {
+        if (lane == 0) flag(a.status, DEV_NOT_SPD);
+        for (int q = lane; q < 5 * nm; q += 32) yv[q] = 0.0;
+        return;
+    }
     __syncwarp();
     // Householder reduction: reflector k stored in column k below the diagonal, tau_k kept; the
     // vector rows are reflected along (y = Q_H^T z). The trailing block is kept in its lower
@@ -191,8 +260,8 @@ __global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
             if (lane == 0) { E[k] = 0.0; P[k] = 0.0; }
             continue;
         }
-        const double alpha = -copysign(sqrt(sigma), x0);
-        const double tau = 1.0 / (alpha * (alpha - x0));
+        const double norm = sigma * rsqrt(sigma), alpha = -copysign(norm, x0);
+        const double tau = 1.0 / fma(fabs(x0), norm, sigma);   // 1 / (alpha (alpha - x0))
         if (lane == 0) A[(k + 1) * ld + k] = x0 - alpha;
         __syncwarp();
         // p = tau A v (rows i > k); the same sweep gives t_q = tau v^T y_q for the vector rows,
