@@ -29,10 +29,12 @@
 // the one that is not to run returns at once.
 //
 // Against an 80-bit recursion (48 columns of 512-atom systems, G at three energies, geometric mean
-// of the relative errors; FP64 kernel first): displaced diamond 7.7e-15 / 7.8e-15 with two classical
-// passes and 8.7e-15 / 7.3e-15 with the second from S'; dense disordered carbon 1.11e-14 / 1.06e-14
-// and 1.19e-14 / 1.20e-14; the same H and S as a caller's: 8.3e-15 / 8.5e-15, 7.9e-15 / 7.1e-15,
-// 1.12e-14 / 1.04e-14, 1.04e-14 / 1.06e-14.
+// of the relative errors; FP64 kernel first, both with the same eigensolver but for its chase):
+// displaced diamond 7.7e-15 / 8.9e-15 with two classical passes and 8.7e-15 / 8.3e-15 with the second
+// from S'; dense disordered carbon 1.11e-14 / 1.40e-14 and 1.19e-14 / 1.40e-14; the same H and S as a
+// caller's: 8.3e-15 / 8.0e-15, 7.9e-15 / 8.7e-15, 1.12e-14 / 1.30e-14, 1.04e-14 / 1.25e-14. Whole density
+// matrices of 512 atoms against dense 64-bit references, mean of eight: 4.7e-15 / 4.9e-15; G: 3.1e-13 /
+// 2.3e-13.
 #include <algorithm>
 
 #include "krylov.cuh"
@@ -359,10 +361,12 @@ __device__ __forceinline__ int2 fx_hi(const int4& v) { return make_int2(v.z, v.w
 // reaches the next shell of the cluster with amplitudes far below the vector's largest (2^-18
 // two bonds on), which FP64 holds to 53 bits of themselves and the integers only to 2^-57 of the
 // largest; where the cluster has a high, localised state there, the later steps amplify what was
-// lost (one column of 16384 in the 4096-atom diamond: its pole at 41.7 eV off by 2e-9 eV, FP64
-// 5e-11, with three such steps 1e-10). After three steps every shell is within 2^-5 of the largest.
-// The vectors are sparse then; the steps cost 4% of the kernel.
-constexpr int kLead = 3;
+// lost. Poles of such columns against an 80-bit recursion, in eV, with 3, 5, 6 and 8 steps in FP64:
+// a 65 eV state of a close pair in disordered carbon 2e-10, 1e-11, 7e-12, 1e-11 (FP64 throughout
+// 6e-12); a state of weight 1e-5 at the rim of a graphite cluster 3e-9, 1.5e-9, 2e-10, 2e-10. Density
+// matrices are on a par with FP64's from five on. Six steps: each costs 3% of the kernel (4096 atoms: 28
+// ms without, 29.8 with 3, 32.8 with 6, 34.9 with 8).
+constexpr int kLead = 6;
 
 template <int T, int kMinB>
 struct FxTmem {
@@ -571,7 +575,7 @@ __device__ __forceinline__ void fx_products(FxState<NC>& st) {
 // The same with dense 4 x 4 blocks, the on-site ones among the entries: 32 products an entry instead of
 // 16, 256 bytes of it instead of 96, which L2 has to deliver. H's block is applied while S's is on its
 // way, and S's while the next entry's H is. 512 atoms, nu 30, set_hs to density matrix: 27.9 ms with the
-// FP64 kernel, 11.7 ms (Slater-Koster form: 11.0 ms).
+// FP64 kernel, 11.9 ms (Slater-Koster form: 11.0 ms).
 template <int NC, int T>
 __device__ __forceinline__ void fx_products_dense(FxState<NC>& st) {
     constexpr int G = T / NC;
