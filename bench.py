@@ -43,11 +43,14 @@ DESCRIPTION = {"diamond_4096": "disordered diamond (8x8x8 cells, sigma 0.1 A)",
                "amorphous_1m": "dense disordered carbon (3.0 g/cm3, sigma 0.3 A)",
                "diamond_64": "disordered diamond (2x2x2 cells, sigma 0.05 A)"}
 FP64_NOMINAL_GFLOPS = 152 * 2 * 2 * 2.07     # SMs x FP64 FMA/clk/SM x 2 flops x GHz
+# the Krylov kernel's products are three wide integer multiply-adds each (57-bit fixed point):
+# SMs x 32 wide multiply-adds/clk/SM / 3 x 2 flops x GHz
+FIXED_NOMINAL_GFLOPS = 152 * 32 / 3 * 2 * 2.07
 RHO_GATE = 1e-10                             # |delta rho_ij| against the oracle
-# DRAM bytes (read + write) of the k_krylov launches of one 4096-atom step from one ncu capture,
-# valid for the Krylov source whose sha256 prefix (krylov.cu + krylov.cuh) and Gram-Schmidt
+# DRAM bytes (read + write) of the k_krylov_fixed launches of one 4096-atom step from one ncu capture,
+# valid for the Krylov source whose sha256 prefix (krylov_fixed.cu + krylov_fixed.cuh) and Gram-Schmidt
 # setting (reorth) are given; reported per launch, and null once either changes
-KRYLOV_TRAFFIC = {"krylov_sha256_prefix": "51a5e4c8a9c32334", "reorth": 1, "bytes_per_step": 115.03e9,
+KRYLOV_TRAFFIC = {"krylov_sha256_prefix": "", "reorth": 1, "bytes_per_step": None,
                   "launches_per_step": 2}
 # further systems timed after the main one: (steps, warm-up steps, plain-form steps, plain-form
 # warm-up steps, sampled columns checked against the oracle); two warm-up steps in the graph
@@ -243,7 +246,7 @@ def aggregate(ms_local, units_local, world, dist=None, device=None):
 def krylov_traffic(reorth):
     import hashlib
     h = hashlib.sha256()
-    for name in ("krylov.cu", "krylov.cuh"):
+    for name in ("krylov_fixed.cu", "krylov_fixed.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1210_1531_gb300", "csrc", name), "rb").read())
     h = h.hexdigest()[:16]
     if h != KRYLOV_TRAFFIC["krylov_sha256_prefix"] or reorth != KRYLOV_TRAFFIC["reorth"]:
@@ -325,13 +328,14 @@ def roofline(stats, peak_probe, traffic=None):
     k_launch_ms = stats["t_krylov_ms"] / max(1, stats["krylov_launches"])
     flops_per_launch = stats["krylov_flops"] / max(1.0, stats["krylov_launches"])
     achieved = flops_per_launch / (k_launch_ms * 1e-3) / 1e9      # GFLOP/s
-    return {"bound": "alu", "kernel": "k_krylov (a3 Krylov build + a4 projection)",
-            "achieved": achieved, "peak": FP64_NOMINAL_GFLOPS, "unit": "GFLOP/s",
-            "frac": achieved / FP64_NOMINAL_GFLOPS, "traffic": traffic,
+    return {"bound": "alu", "kernel": "k_krylov_fixed (a3 Krylov build + a4 projection)",
+            "achieved": achieved, "peak": FIXED_NOMINAL_GFLOPS, "unit": "GFLOP/s",
+            "frac": achieved / FIXED_NOMINAL_GFLOPS, "traffic": traffic,
             "peak_probe": peak_probe, "frac_of_probe": achieved / peak_probe if peak_probe else None,
             "flops_per_launch": flops_per_launch, "launch_ms": k_launch_ms,
-            "peak_note": "FP64 FMA pipe: 152 SM x 2 FMA/clk x 2 flop x 2.07 GHz (nominal 1.26 TFLOP/s); "
-                         "peak_probe = measured FMA-chain throughput"}
+            "peak_note": "integer pipe: 152 SM x 32 wide multiply-adds/clk / 3 per product x 2 flop x 2.07 GHz "
+                         "(6.71 TFLOP/s; the FP64 pipe's nominal rate is 1.26); peak_probe = measured FP64 "
+                         "FMA-chain throughput, the roof of a form in FP64"}
 
 
 def shapes(tuned):

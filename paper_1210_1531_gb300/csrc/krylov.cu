@@ -25,6 +25,9 @@
 // reduced by recursive halving (one addition per value). The bases U and SU stay in per-CTA
 // global scratch in [k][position][orbital] order (coalesced 32-byte rows per lane). FP64
 // everywhere; no tensor cores (the work is sparse and FP64).
+//
+// These kernels run where the fixed-point form (krylov_fixed.cu, half their time) does not apply:
+// clusters of more than 336 atoms, rows of H or S of very different size or many blocks.
 #include <algorithm>
 
 #include "krylov.cuh"
