@@ -50,7 +50,7 @@ RHO_GATE = 1e-10                             # |delta rho_ij| against the oracle
 # DRAM bytes (read + write) of the k_krylov_fixed launches of one 4096-atom step from one ncu capture,
 # valid for the Krylov source whose sha256 prefix (krylov_fixed.cu + krylov_fixed.cuh) and Gram-Schmidt
 # setting (reorth) are given; reported per launch, and null once either changes
-KRYLOV_TRAFFIC = {"krylov_sha256_prefix": "", "reorth": 1, "bytes_per_step": None,
+KRYLOV_TRAFFIC = {"krylov_sha256_prefix": "ef237440b472bcb8", "reorth": 1, "bytes_per_step": 11.17e9,
                   "launches_per_step": 2}
 # further systems timed after the main one: (steps, warm-up steps, plain-form steps, plain-form
 # warm-up steps, sampled columns checked against the oracle); two warm-up steps in the graph
