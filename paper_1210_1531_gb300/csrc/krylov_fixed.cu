@@ -1375,6 +1375,12 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
                 const int warp = threadIdx.x >> 5;
                 const bool idle = warp >= 2 * NC || st.done[warp % NC];   // (done changes below)
                 __syncthreads();
+                // the magnitudes were last read before pass A; the update's, of every warp, come after
+                // the barrier below
+                if (threadIdx.x < NC) {
+                    st.bits[0][threadIdx.x] = st.bits[1][threadIdx.x] = 0;
+                    st.top[0][threadIdx.x] = st.top[1][threadIdx.x] = 0;
+                }
                 if (!idle && warp < NC) fx_scalars<NC>(a, st, n, warp);
                 else if (!idle) fx_scalars_h<NC>(a, st, n, warp - NC);
                 __syncthreads();
@@ -1383,11 +1389,7 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
                     __syncthreads();
                 }
                 for (int q = threadIdx.x; q < 3 * NC * (3 * st.nm + 1); q += T) fx_at<int>(st.v.red)[q] = 0;
-                if (threadIdx.x < NC) {
-                    st.bits[0][threadIdx.x] = st.bits[1][threadIdx.x] = 0;
-                    st.top[0][threadIdx.x] = st.top[1][threadIdx.x] = 0;
-                    st.we[threadIdx.x] = 0;
-                }
+                if (threadIdx.x < NC) st.we[threadIdx.x] = 0;   // read and written by this thread until the next step
                 if (st.live == 0) {
                     __syncthreads();   // st.live is set again for the next columns
                     break;
