@@ -117,7 +117,7 @@ int prepare_columns(elses_system s) {
     // warps per SM as k_krylov at capacity 16 (c + 1), or as the autotuner chose; the others run
     // k_krylov. Otherwise slots of 32.
     const bool half_ok = s->p.k3_lanes != 32 && s->p.force_mode == 0 && !s->p.krylov_block;
-    const bool fx_ok = s->fx && !s->user_hs && !s->p.krylov_block;
+    const bool fx_ok = s->fx && s->fx_room(false) && !s->user_hs && !s->p.krylov_block;
     const int gslot = half_ok ? 16 : 32;
     std::vector<int> ord;
     ord.reserve(s->n);
@@ -168,7 +168,7 @@ int prepare_columns(elses_system s) {
             bps = shape(false, bps, bps_max);
             const int bps64 = bps, grid64 = std::min(count, s->num_sms * bps);
             if (fx_b > 0) {
-                fx_dense = form;
+                if (s->fx_room(true)) fx_dense = form;
                 if (fx_ok) fx = form;
             }
             if (fx >= 0) bps = shape(true, fx_b, fx_b);
@@ -176,7 +176,7 @@ int prepare_columns(elses_system s) {
             s->k3_launches.push_back({b, e, begin, count, na, grid, bps, half ? 1 : 0, key, fx, fx_dense, grid64, bps64, batch_off});
             // scratch for the kernel with the largest need, as caller matrices change it without a new plan
             const size_t fp64 = (size_t)grid64 * kWarpsPerAtom * 2 * nm * na * 4;
-            const size_t fixed = fx_dense >= 0 ? (size_t)std::min(fx_items(form, count), s->num_sms * fx_b) * fx_scratch_doubles(form, nm, na) : 0;
+            const size_t fixed = fx >= 0 || fx_dense >= 0 ? (size_t)std::min(fx_items(form, count), s->num_sms * fx_b) * fx_scratch_doubles(form, nm, na) : 0;
             batch_off += s->p.krylov_block ? (size_t)grid * block_krylov_scratch_doubles(nm, na) : std::max(fp64, fixed);
             scratch = std::max(scratch, batch_off);
             if (count > best_items) { best_items = count; s->k3_bps = bps; }
@@ -446,7 +446,11 @@ int ensure_V(elses_system s, cudaStream_t st) {
 
 void launch_krylov(elses_system s, const KrylovArgs& ka, int fx, int grid, int bps, cudaStream_t st) {
     if (s->p.krylov_block) block_krylov_columns(ka, grid, st);
-    else if (fx >= 0) fx_columns(ka, FxArgs{reinterpret_cast<const int4*>(s->fx_rec.p), s->fx_scale.p, s->skd.Es, s->skd.Ep, 0, 0}, fx, grid, bps, st);
+    else if (fx >= 0) {
+        const bool caller = ka.skr == nullptr;
+        const int2* rec = caller ? s->fxu_rec.p : s->fx_rec.p;
+        fx_columns(ka, FxArgs{reinterpret_cast<const int4*>(rec), s->fx_scale.p + (caller ? 1 : 0), s->skd.Es, s->skd.Ep, 0, 0}, fx, grid, bps, st);
+    }
     else krylov_columns(ka, grid, bps, st);
 }
 
@@ -508,7 +512,7 @@ int run_batch(elses_system s, int b, int e, bool stored, double** V_out, int* v_
             const int bps = s->p.k3_ctas_per_sm > 0 ? std::min(fb, s->p.k3_ctas_per_sm) : fb;
             launch_krylov(s, ka, L.fx_dense, std::min(fx_items(L.fx_dense, L.item_count), s->num_sms * bps), bps, lst);
             s->stats.launches++;
-            ka.skip = &s->fx_scale.p->ok;
+            ka.skip = &s->fx_scale.p[1].ok;
         }
         if (s->user_hs) launch_krylov(s, ka, -1, L.grid64, L.bps64, lst);
         else launch_krylov(s, ka, L.fx, L.grid, L.bps, lst);
@@ -788,6 +792,24 @@ int energy_force_eager(elses_system s, double* mu_host, double* e_band_host, dou
     return warn > 0 ? warn : rc;
 }
 
+// Room for the records of the fixed-point kernel's blocks, 96 bytes a block for the Slater-Koster form and
+// 256 for a caller's matrices. Both with the pattern, so that elses_set_hs allocates nothing: it may be
+// captured, as may any other stream. Where the memory is not there the FP64 kernels run instead.
+static void reserve_records(elses_system s) {
+    if (s->p.krylov_block) return;
+    s->fx_rec.try_ensure(12 * (size_t)s->nnzb);
+    s->fxu_rec.try_ensure(32 * (size_t)s->nnzb);
+}
+
+// The plan; without the records, and so with the FP64 kernels' scratch only, where memory does not reach.
+static int prepare_with_records(elses_system s) {
+    const int rc = prepare_columns(s);
+    if (rc != ELSES_ERR_OOM || !(s->fx_rec.p || s->fxu_rec.p)) return rc;
+    s->fxu_rec.release();
+    s->fx_rec.release();
+    return prepare_columns(s);
+}
+
 }  // namespace elses
 
 extern "C" {
@@ -1011,18 +1033,20 @@ int elses_build_clusters(elses_system* sys, int n_atoms, const double* pos_dev,
     sk_build(s->pos.p, n, s->box, s->skd, s->row_ptr.p, s->col_idx.p, s->nnzb, s->row_of.p, s->tmap.p,
              s->H.p, s->S.p, s->skr.p, st);
     s->stats.launches += 2;
-    TRY(s->fx_rec.ensure((size_t)s->nnzb * 12));
-    TRY(s->fx_scale.ensure(1));
-    TRY(s->fx_bounds.ensure(6));
-    fx_build(n, s->nnzb, s->row_ptr.p, s->col_idx.p, s->skr.p, s->skd.Es, s->skd.Ep, s->max_nb, s->fx_bounds.p,
-             s->fx_scale.p, s->fx_rec.p, st);
-    s->stats.launches += 3;
+    reserve_records(s);
+    TRY(s->fx_scale.ensure(2));
+    TRY(s->fx_bounds.ensure(12));
     int fx_ok = 0;
-    CUDA_TRY(cudaMemcpyAsync(&fx_ok, &s->fx_scale.p->ok, sizeof(int), cudaMemcpyDeviceToHost, st));
+    if (s->fx_room(false)) {
+        fx_build(n, s->nnzb, s->row_ptr.p, s->col_idx.p, s->skr.p, s->skd.Es, s->skd.Ep, s->max_nb, s->fx_bounds.p,
+                 s->fx_scale.p, s->fx_rec.p, st);
+        s->stats.launches += 3;
+        CUDA_TRY(cudaMemcpyAsync(&fx_ok, &s->fx_scale.p->ok, sizeof(int), cudaMemcpyDeviceToHost, st));
+    }
     if (clusters) TRY(join_side(s, st));   // the cluster lists
     TRY(check_status(s, st));
     s->fx = fx_ok != 0;
-    TRY(prepare_columns(s));
+    TRY(prepare_with_records(s));
     if (s->p.autotune && s->tuned_bps.empty() && s->p.k3_ctas_per_sm <= 0) TRY(autotune_impl(s, st));
     return ELSES_OK;
 }
@@ -1101,19 +1125,20 @@ int elses_set_hs(elses_system s, int nnzb, const int* row_ptr_dev, const int* co
         TRY(adopt_pattern(s, nnzb, row_ptr_dev, col_idx_dev, st));   // checks before it changes anything
         s->user_hs = true;
         s->drop_graph();
-        TRY(prepare_columns(s));
+        reserve_records(s);
+        TRY(prepare_with_records(s));
     }
     s->user_hs = true;
     CUDA_TRY(cudaMemcpyAsync(s->H.p, H_dev, sizeof(double) * 16 * s->nnzb, cudaMemcpyDeviceToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(s->S.p, S_dev, sizeof(double) * 16 * s->nnzb, cudaMemcpyDeviceToDevice, st));
-    // records for the fixed-point kernel (their buffer is not allocated while the stream is captured)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-    s->fx_user = !s->p.krylov_block && (cap == cudaStreamCaptureStatusNone || s->fx_rec.cap >= 32 * (size_t)s->nnzb);
+    // The fixed-point kernel's records and the device's choice of kernel follow the values that this call,
+    // or a replay of it where it is captured, writes.
+    s->fx_user = s->fx_room(true);
     if (s->fx_user) {
-        TRY(s->fx_rec.ensure(32 * (size_t)s->nnzb));
-        fx_build_dense(s->n, s->nnzb, s->row_ptr.p, s->H.p, s->S.p, s->max_nb, s->fx_bounds.p, s->fx_scale.p, s->fx_rec.p, st);
+        fx_build_dense(s->n, s->nnzb, s->row_ptr.p, s->H.p, s->S.p, s->max_nb, s->fx_bounds.p + 6, s->fx_scale.p + 1, s->fxu_rec.p, st);
         s->stats.launches += 3;
+    } else {
+        CUDA_TRY(cudaMemsetAsync(&s->fx_scale.p[1].ok, 0, sizeof(int), st));
     }
     s->have_rho = false;
     s->v_lazy = false;   // every column is recomputed before V is used again

@@ -48,7 +48,7 @@ extern unsigned long long g_alloc_epoch;
 template <class T>
 struct DevBuf {
     T* p = nullptr;
-    size_t cap = 0;
+    size_t cap = 0, refused = 0;
     int ensure(size_t n) {
         if (n <= cap && p) return 0;
         if (p) cudaFree(p);
@@ -62,6 +62,14 @@ struct DevBuf {
         cap = want;
         ++g_alloc_epoch;
         return 0;
+    }
+    // the same without an error: false where the memory is not there (asked for again only when more is needed)
+    bool try_ensure(size_t n) {
+        if ((n <= cap && p) || n <= refused) return n <= cap && p;
+        release();
+        if (ensure(n) >= 0) return true;
+        refused = n;
+        return false;
     }
     void release() {   // a captured graph that used the buffer is then out of date
         if (p) {
@@ -116,9 +124,14 @@ struct elses_system_s {
     };
     bool fx = false;                       // the fixed-point Krylov form suits the system's H and S
     bool fx_user = false;                  // caller matrices have records (fx_scale->ok says whether they are used)
-    DevBuf<elses::FxScale> fx_scale;
-    DevBuf<unsigned long long> fx_bounds;
-    DevBuf<int2> fx_rec;
+    DevBuf<elses::FxScale> fx_scale;       // of the Slater-Koster system, of the caller's matrices
+    DevBuf<unsigned long long> fx_bounds;  // 6 words each
+    DevBuf<int2> fx_rec, fxu_rec;          // block records likewise
+    // whether the records of the Slater-Koster form, or of the caller's, have their room
+    bool fx_room(bool caller) const {
+        const DevBuf<int2>& r = caller ? fxu_rec : fx_rec;
+        return !p.krylov_block && r.p && r.cap >= (caller ? 32 : 12) * (size_t)nnzb;
+    }
     cudaStream_t side = nullptr;           // second stream for concurrent class launches
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<K3Launch> k3_launches;
