@@ -56,6 +56,7 @@ __global__ void k_fx_bounds(int n, const int* __restrict__ row_ptr, const int* _
         v[3] = 1.0;
         v[0] = v[2];
         v[1] = 1.0;
+        bool finite = isfinite(Es) && isfinite(Ep);   // (fmax drops a NaN)
         for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
             if (col_idx[e] == i) continue;
             const double* q = skr + 12 * (size_t)e;
@@ -64,10 +65,14 @@ __global__ void k_fx_bounds(int n, const int* __restrict__ row_ptr, const int* _
                 const double pi = fabs(q[6 + 4 * m]), dv = fabs(q[7 + 4 * m]);
                 v[m] += fmax(ss, pi) + 1.75 * (sp + dv);
                 v[2 + m] = fmax(v[2 + m], fmax(fmax(ss, sp), fmax(pi, dv)));
-                // NaN and infinities (fmax drops a NaN): recorded as the largest value
-                if (!(ss + sp + pi + dv <= 1e300)) v[m] = v[2 + m] = 1e308;
+                finite = finite && ss + sp + pi + dv <= 1e300;
             }
+            // u: the direction, not a number between atoms in one place
+            const double* u = skr + 12 * (size_t)e;
+            finite = finite && fabs(u[0]) + fabs(u[1]) + fabs(u[2]) <= 2.0;
         }
+        // NaN and infinities are recorded as the largest value: the FP64 kernels then run and report them
+        if (!finite) v[0] = v[1] = v[2] = v[3] = 1e308;
     }
     unsigned long long w[6];
     for (int m = 0; m < 4; ++m) w[m] = (unsigned long long)__double_as_longlong(v[m]);
