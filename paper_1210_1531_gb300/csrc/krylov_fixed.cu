@@ -100,6 +100,8 @@ __global__ void k_fx_scale(const unsigned long long* b, double Es, double Ep, in
     s.ok = max_row <= (dense ? 32 : 64);
     for (int m = 0; m < 2; ++m)
         if (!(v[m] > 1e-100 && v[m] < 1e100 && v[m] <= 256.0 * lo[m] && v[2 + m] > 0.0)) s.ok = 0;
+    // the second Gram-Schmidt pass takes its coefficients, of order 2^63 sqrt(S), to single precision
+    if (!(v[1] > 0x1p-60 && v[1] < 0x1p60)) s.ok = 0;
     if (s.ok) {
         const int row_bits = max_row <= 32 ? 61 : 59;
         s.eH = min(56 + dense - ilogb(v[2]), row_bits - ilogb(v[0]));
