@@ -228,14 +228,28 @@ __global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
     const double* Sp = a.Sp + (size_t)c * PK;
 
     bool unit = true;      // S' = I to 2^-32
+    unsigned top[4] = {0u, 0u, 0u, 0u};   // upper words of the largest |H'|, |U_j|, |SU_j| and |HU_j|
     for (int q = lane; q < nu * nu; q += 32) {
         const int i = q / nu, k = q % nu;
-        const double s = packed(Sp, i, k);
-        A[i * ld + k] = packed(Hp, i, k);
+        const double s = packed(Sp, i, k), h = packed(Hp, i, k);
+        A[i * ld + k] = h;
         L[i * ld + k] = s;
         unit = unit && fabs(i == k ? s - 1.0 : s) < 0x1p-32;
+        top[0] = max(top[0], (unsigned)__double2hiint(h) & 0x7fffffffu);
+    }
+    for (int k = lane; k < nu; k += 32) {
+        const size_t at = (size_t)c * nm + k;
+        top[1] = max(top[1], (unsigned)__double2hiint(a.urow[at]) & 0x7fffffffu);
+        top[2] = max(top[2], (unsigned)__double2hiint(a.surow[at]) & 0x7fffffffu);
+        top[3] = max(top[3], (unsigned)__double2hiint(a.hurow[at]) & 0x7fffffffu);
     }
     unit = __all_sync(0xffffffffu, unit);
+    // and magnitudes that FP32 holds with what is 2^-56 of them: the largest zero, or 2^-60 to 2^100
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        top[q] = __reduce_max_sync(0xffffffffu, top[q]);
+        unit = unit && (top[q] == 0u || (top[q] >= (1023u - 60u) << 20 && top[q] < (1023u + 100u) << 20));
+    }
     __syncwarp();
     if (unit) {
         reduce_unit(A, L, P, nu, ld, lane, a.urow + (size_t)c * nm, a.surow + (size_t)c * nm, a.hurow + (size_t)c * nm);

@@ -24,3 +24,10 @@ def _poles(h_exp, s_exp, reorth):
 def test_scaled_overlap(s_exp, reorth):
     want = _poles(0, 0, reorth)
     assert float((_poles(0, s_exp, reorth) - want).abs().max()) <= 1e-12 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("h_exp", [-300, -140, -70, 90, 126, 140, 300])
+@pytest.mark.parametrize("reorth", [0, 1])
+def test_scaled_hamiltonian(h_exp, reorth):
+    want = _poles(0, 0, reorth)
+    assert float((_poles(h_exp, 0, reorth) - want).abs().max()) <= 1e-12 * float(want.abs().max())
