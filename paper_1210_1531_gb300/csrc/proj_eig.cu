@@ -363,11 +363,12 @@ __global__ void __launch_bounds__(kChaseThreads) k_eig_chase(const EigArgs a) {
     const size_t cap = eig_rot_cap(nm);
     size_t nrot = 0;
     bool ok = true;
-    // |E_k| <= 2^-52 max(|D_k|, |D_k+1|), to the last of the 20 mantissa bits of their upper words
+    // |E_k| <= 2^-52 max(|D_k|, |D_k+1|), to the last of the 20 mantissa bits of their upper words. False
+    // where one is not a number, as the comparison of the numbers would be: the sweep cap then ends the chase.
     auto negligible = [&](int k) {
         const int e = __double2hiint(E[k]) & 0x7fffffff;
         const int d = max(__double2hiint(D[k]) & 0x7fffffff, __double2hiint(D[k + 1]) & 0x7fffffff);
-        return e == 0 || e + (52 << 20) <= d;
+        return d <= 0x7ff00000 && (e == 0 || e <= d - (52 << 20));
     };
     int hi = nu - 1, sweeps = 0;
     const int max_sweeps = a.max_sweeps > 0 ? a.max_sweeps : 30 * nu;
