@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "elses.h"
 
 namespace elses {
@@ -25,9 +27,12 @@ constexpr int kWarpsPerAtom = 4;    // one warp per orbital column of an atom
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` and never lowers it: the limit
 // is a property of the function, shared by every system on the device, and after the first
 // launches no attribute call stays on the launch path (where it could order launches that are
-// meant to overlap).
+// meant to overlap). Looked at and raised under a lock: of two threads that find it too low, the
+// later must not set the smaller limit.
 template <typename Kernel>
 inline void smem_at_least(Kernel kernel, size_t bytes) {
+    static std::mutex one_at_a_time;
+    const std::lock_guard<std::mutex> hold(one_at_a_time);
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, kernel) == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);

@@ -1482,11 +1482,7 @@ void fx_columns(const KrylovArgs& a, FxArgs x, int form, int grid, int ctas_per_
     x.smem_bytes = (int)(std::min(all, share) & ~(size_t)15);
     x.split = f.nc < 4;
     const void* fn = a.skr ? f.fn : f.fn_dense;
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess || fa.maxDynamicSharedSizeBytes < x.smem_bytes) {
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, x.smem_bytes);
-        cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    }
+    smem_at_least(fn, kSmemCta - kSmemStatic);   // what any launch of it may ask for
     void* args[] = {const_cast<KrylovArgs*>(&a), &x};
     cudaLaunchKernel(fn, dim3(grid), dim3(f.t), args, (size_t)x.smem_bytes, st);
 }
