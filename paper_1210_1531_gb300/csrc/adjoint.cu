@@ -38,11 +38,12 @@
 //  associative, so the sums, and the gradient and forces after them, are the same bit for bit
 //  whatever the order in which the CTAs arrive. One pass at the end converts them to FP64.
 //
-// The bases come from the energy pass when it kept them (the Krylov kernel's store form),
-// otherwise the forward recursion is recomputed here by the Krylov kernel's own code
-// (column_forward with kAdj: it also keeps HU and the Gram-Schmidt coefficients); V, e, c, d
-// come from the columns already computed for the same positions. One CTA of 4 warps per atom; the lanes own cluster
-// rows as in the Krylov kernel; the bases and factors live in per-warp global scratch.
+// The bases, HU, H' and the Gram-Schmidt coefficients are those the Krylov kernel kept (its store form),
+// in the energy pass where all columns' fit in memory, otherwise in a second launch of the same kernel
+// over the items that the next launch of this one takes: the recursion is the one that V, e, c, d come
+// from, bit for bit. (Recomputed in other arithmetic, a nearly exhausted space gives other bases, and the
+// gradient was off by up to 5e-5.) One CTA of 4 warps per atom; the lanes own cluster rows as in k_krylov;
+// the factors live in per-warp global scratch.
 #include "krylov.cuh"
 
 namespace elses {
@@ -117,23 +118,21 @@ __device__ __forceinline__ double packed_at(const double* P, int i, int k) {
 }
 
 struct WarpScratch {
-    double *U, *SU, *HU, *Ub, *YH, *YS, *T;        // vectors: nm x (NA x 4) each, T: NA x 4
-    double *hess, *X, *Tm, *Hh, *Sg, *Sy;           // nm x nm each
+    double *U, *SU, *HU, *hess;                     // of the kept column
+    double *Ub, *YH, *YS, *T;                       // vectors: nm x (NA x 4) each, T: NA x 4
+    double *X, *Tm, *Hh, *Sg, *Sy;                  // nm x nm each
     double *om, *abar, *bbar;                      // nm each
 };
 
 __device__ __forceinline__ WarpScratch warp_scratch(double* base, int nm, int NA) {
     WarpScratch w;
     const size_t vsz = (size_t)nm * NA * 4, mm = (size_t)nm * nm;
-    w.U = base;
-    w.SU = w.U + vsz;
-    w.HU = w.SU + vsz;
-    w.Ub = w.HU + vsz;
+    w.U = w.SU = w.HU = w.hess = nullptr;
+    w.Ub = base;
     w.YH = w.Ub + vsz;
     w.YS = w.YH + vsz;
     w.T = w.YS + vsz;
-    w.hess = w.T + (size_t)NA * 4;
-    w.X = w.hess + mm;
+    w.X = w.T + (size_t)NA * 4;
     w.Tm = w.X + mm;
     w.Hh = w.Tm + mm;
     w.Sg = w.Hh + mm;
@@ -376,7 +375,7 @@ __device__ __forceinline__ void sampled_block(const AdjointArgs& g, const int* n
 }  // namespace
 
 __host__ __device__ size_t adjoint_warp_doubles(int nm, int na_max) {
-    const size_t d = 6 * (size_t)nm * na_max * 4 + (size_t)na_max * 4 + 6 * (size_t)nm * nm + 3 * (size_t)nm;
+    const size_t d = 3 * (size_t)nm * na_max * 4 + (size_t)na_max * 4 + 5 * (size_t)nm * nm + 3 * (size_t)nm;
     return (d + 3) & ~(size_t)3;   // keeps every warp's area 32-byte aligned
 }
 
@@ -390,7 +389,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_adjoint(const KrylovArgs a, con
     double* hbuf = vec + (size_t)kWarpsPerAtom * 2 * NA * 4;
     ClusterView v;
     carve_view(reinterpret_cast<unsigned char*>(hbuf + kWarpsPerAtom * kMaxNu), NA, a.deg_max, v);
-    __shared__ int sh_atom, sh_nv[kWarpsPerAtom];
+    __shared__ int sh_atom, sh_slot, sh_nv[kWarpsPerAtom];
     __shared__ const double* sh_U[kWarpsPerAtom];
     __shared__ const double* sh_YH[kWarpsPerAtom];
     __shared__ const double* sh_YS[kWarpsPerAtom];
@@ -408,9 +407,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_adjoint(const KrylovArgs a, con
                 if (atom < g.atom_lo || atom >= g.atom_hi) atom = -2;   // outside the requested atoms
             }
             sh_atom = atom;
+            sh_slot = a.again ? idx : atom;
         }
         __syncthreads();
-        const int J = sh_atom;
+        const int J = sh_atom, slot = sh_slot;
         if (J == -1) break;
         if (J < 0) {
             __syncthreads();
@@ -429,31 +429,18 @@ __global__ void __launch_bounds__(kThreads, 3) k_adjoint(const KrylovArgs a, con
             double* A = vec + (size_t)(warp * 2) * NA * 4;
             double* B = A + (size_t)NA * 4;
             double* hb = hbuf + warp * kMaxNu;
-            int jp = 0;
-            const double* Hpc;
-            if (g.bstore) {   // the bases the energy pass kept
-                const int aJ = bsearch_sorted(v.cl, v.n_at, J);
-                nv = aJ >= 0 ? a.nu_eff[j] : 0;
-                if (nv <= 0) {
-                    nv = 0;
-                    break;
-                }
-                jp = 4 * v.pos_of[aJ] + alpha;
-                double* col = const_cast<double*>(g.bstore) + (size_t)j * g.bstride;
-                w.U = col;
-                w.SU = col + g.bvec;
-                w.HU = col + 2 * g.bvec;
-                w.hess = col + 3 * g.bvec;
-                Hpc = w.hess + (size_t)nm * nm;
-            } else {
-                int nu = 0;
-                nv = column_forward<true>(a, v, J, alpha, A, B, hb, w.U, w.SU, w.HU, w.hess, nu, jp);
-                if (nv <= 0) {
-                    nv = 0;
-                    break;
-                }
-                Hpc = a.Hp + (size_t)(j - 4 * a.atom_begin) * (nm * (nm + 1) / 2);
+            const int aJ = bsearch_sorted(v.cl, v.n_at, J);
+            nv = aJ >= 0 ? min(a.nu_eff[j], g.nu_kept[j]) : 0;   // (V has a.nu_eff rows)
+            if (nv <= 0) {
+                nv = 0;
+                break;
             }
+            const int jp = 4 * v.pos_of[aJ] + alpha;
+            w.U = a.bstore + (size_t)(4 * slot + alpha) * a.bstride;
+            w.SU = w.U + a.bvec;
+            w.HU = w.SU + a.bvec;
+            w.hess = w.HU + a.bvec;
+            const double* Hpc = w.hess + (size_t)nm * nm;
             __syncwarp();
             const double sq = 1.0 / w.U[jp];                   // sqrt(S_jj): u_1 = e_j / sqrt(S_jj)
             rayleigh_ritz_gradient(g, g.V + (size_t)(j - g.v_col0) * nm * nm, g.eps + (size_t)j * nm,
@@ -495,8 +482,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_adjoint(const KrylovArgs a, con
             const unsigned long long blocks = nent + (onsite ? nat : 0ull);
             unsigned long long f = 8ull * vv * vv * nc + 6ull * vv * vv * vv + 64ull * vv * blocks;
             f += (vv - 1) * (8ull * nc + per * nent + (onsite ? 4ull * nat : 0ull)) + 5ull * nc * vv * (vv - 1);
-            if (!g.bstore)   // the forward recursion recomputed: the Krylov kernel's count
-                f += column_flops(a, v.n_at, v.nent, nv, a.reorth != 0);
             atomicAdd(g.flops, f);
         }
         if (lane == 0) {

@@ -104,10 +104,14 @@ struct KrylovArgs {
     // Gram-Schmidt coefficients [nu_max][nu_max] and H' packed upper
     double* bstore;
     size_t bstride, bvec;
+    // the columns built once more for the gradient (0 in the energy pass): the store holds this launch's
+    // items, column alpha of item q at 4 q + alpha, of the atoms [only_lo, only_hi) alone, and a
+    // space that ends early was reported before
+    int again, only_lo, only_hi;
 };
 
-// Exact-gradient pass (adjoint.cu) over the columns of a batch; the KrylovArgs of the same batch
-// drive the recomputed forward recursion.
+// Exact-gradient pass (adjoint.cu) over the columns of a batch, from the bases that the Krylov kernel
+// of the same KrylovArgs kept.
 struct AdjointArgs {
     const double* V;        // [col - v_col0][nu_max][nu_max] eigenvectors (rows: Krylov index)
     int v_col0;
@@ -125,8 +129,7 @@ struct AdjointArgs {
     int* status;
     double* scratch;        // per resident CTA: 4 warps x adjoint_warp_doubles(nu_max, na_max)
     int atom_lo, atom_hi;   // only atoms in [atom_lo, atom_hi) are accumulated
-    const double* bstore;   // bases kept by the energy pass (KrylovArgs layout), or nullptr:
-    size_t bstride, bvec;   // then the forward recursion is recomputed
+    const int* nu_kept;     // [M] steps that were kept of each column
 };
 // fixed-point form (krylov_fixed.cu): scales and block records of a Slater-Koster system (bounds:
 // six words), then the launch of a size class

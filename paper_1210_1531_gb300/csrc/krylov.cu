@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kThreads, kMinB) k_krylov(const KrylovArgs a) 
     double* hbuf = vec + (size_t)kWarpsPerAtom * 2 * NA * 4;
     ClusterView v;
     carve_view(reinterpret_cast<unsigned char*>(hbuf + kWarpsPerAtom * kMaxNu), NA, a.deg_max, v);
-    __shared__ int sh_atom;
+    __shared__ int sh_atom, sh_slot;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const size_t warp_scratch = (size_t)2 * a.nu_max * NA * 4;
@@ -69,11 +69,17 @@ __global__ void __launch_bounds__(kThreads, kMinB) k_krylov(const KrylovArgs a) 
             const int idx = a.queue ? atomicAdd(a.queue, 1) : blockIdx.x + iter * gridDim.x;
             int atom = -1;
             if (idx < n_batch) atom = a.order[idx];
+            if (kStore && a.again && atom >= 0 && (atom < a.only_lo || atom >= a.only_hi)) atom = -2;
             sh_atom = atom;
+            sh_slot = kStore && a.again ? idx : atom;
         }
         __syncthreads();
-        const int J = sh_atom;
-        if (J < 0) break;
+        const int J = sh_atom, slot = sh_slot;
+        if (J == -1) break;
+        if (J < 0) {
+            __syncthreads();
+            continue;
+        }
         if (!cluster_view(a, J, NA, v)) {
             if (tid == 0) flag(a.status, DEV_CAPACITY);
             __syncthreads();
@@ -90,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, kMinB) k_krylov(const KrylovArgs a) 
             int nu = 0, jp = 0;
             double *Ucol = Uw, *SUcol = SUw, *HUcol = nullptr, *hess = nullptr;
             if constexpr (kStore) {
-                Ucol = a.bstore + (size_t)j * a.bstride;
+                Ucol = a.bstore + (size_t)(4 * slot + alpha) * a.bstride;
                 SUcol = Ucol + a.bvec;
                 HUcol = SUcol + a.bvec;
                 hess = HUcol + a.bvec;
@@ -107,7 +113,7 @@ __global__ void __launch_bounds__(kThreads, kMinB) k_krylov(const KrylovArgs a) 
             }
             if (lane == 0) {
                 a.nu_eff[j] = nu_eff;
-                if (nu_eff < nu) flag(a.status, DEV_BREAKDOWN);
+                if (nu_eff < nu && !a.again) flag(a.status, DEV_BREAKDOWN);
                 if (a.flops) atomicAdd(a.flops, column_flops(a, n_at, v.nent, nu_eff, a.reorth != 0));
             }
             __syncwarp();

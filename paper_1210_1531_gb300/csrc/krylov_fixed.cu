@@ -268,6 +268,7 @@ struct FxState {
     int kT, kS, kY;         // U[0, kT) in tensor memory, U[kT, kS) and SU[0, kY) in shared memory
     bool overlap;
     int atom, live;
+    int slot;               // of the atom's columns in the store of bases
     unsigned long long bits[2][NC];   // or of the magnitudes of new vectors
     unsigned top[2][NC];    // the same of the lead's FP64 vectors: largest high word
     int bH[NC], bS[NC];     // H u_n = f 2^bH P, S u_n = f 2^bS Y
@@ -905,7 +906,7 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
             f[n] = fn;
             s[n] = sn;
         }
-        double* hess = a.bstore ? a.bstore + (size_t)(4 * st.atom + st.alpha0 + c) * a.bstride + 3 * a.bvec : nullptr;
+        double* hess = a.bstore ? a.bstore + (size_t)(4 * st.slot + st.alpha0 + c) * a.bstride + 3 * a.bvec : nullptr;
         if (hess && n > 0 && lane == 0)     // beta_(n-1) = |w|_S
             hess[(size_t)(n - 1) * nm + n] = sqrt(xsx * fx_pow2(2 * st.we[c])) *
                                              (f[n - 1] * fx_pow2(fx_at<int>(st.v.ex)[(NC + c) * nm + n - 1]));
@@ -1235,7 +1236,7 @@ __device__ __forceinline__ void fx_keep_step(const KrylovArgs& a, FxState<NC>& s
     for (int q = threadIdx.x; q < np * 4 * NC; q += T) {
         const int r = q & 3, p = (q >> 2) % np, c = (q >> 2) / np, at = pos_atom[p];
         if (n >= st.nue[c]) continue;
-        double* out = a.bstore + (size_t)(4 * st.atom + st.alpha0 + c) * a.bstride + (size_t)n * np * 4 + 4 * p + r;
+        double* out = a.bstore + (size_t)(4 * st.slot + st.alpha0 + c) * a.bstride + (size_t)n * np * 4 + 4 * p + r;
         double u = 0.0, su = 0.0, hu = 0.0;
         if (at >= 0) {
             const int k = 2 * fx_unit<NC>(at, r >> 1, c) + (r & 1);
@@ -1261,7 +1262,7 @@ __device__ __forceinline__ void fx_results(const KrylovArgs& a, FxState<NC>& st,
     if (tid < NC) {
         const int ne = st.nue[tid];
         a.nu_eff[4 * J + alpha0 + tid] = ne;
-        if (ne < nu) flag(a.status, DEV_BREAKDOWN);
+        if (ne < nu && !a.again) flag(a.status, DEV_BREAKDOWN);
         if (a.flops) atomicAdd(a.flops, column_flops(a, st.n_at, st.nent, ne, st.overlap));
     }
     for (int q = tid; q < 3 * NC * nm; q += T) {
@@ -1275,7 +1276,7 @@ __device__ __forceinline__ void fx_results(const KrylovArgs& a, FxState<NC>& st,
         const int PK = nm * (nm + 1) / 2;
         for (int q = tid; q < NC * PK; q += T) {
             const int c = q / PK, k = q % PK;
-            a.bstore[(size_t)(4 * J + alpha0 + c) * a.bstride + 3 * a.bvec + (size_t)nm * nm + k] = a.Hp[(col0 + c) * PK + k];
+            a.bstore[(size_t)(4 * st.slot + alpha0 + c) * a.bstride + 3 * a.bvec + (size_t)nm * nm + k] = a.Hp[(col0 + c) * PK + k];
         }
     }
     if (a.UP) {
@@ -1336,8 +1337,10 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
         if (threadIdx.x == 0) {
             const int item = a.queue ? atomicAdd(a.queue, 1) : blockIdx.x + iter * gridDim.x;
             const int idx = x.split ? item / (4 / NC) : item;
-            const int J = idx < a.n_items ? a.order[idx] : -1;
+            int J = idx < a.n_items ? a.order[idx] : -1;
+            if (a.again && J >= 0 && (J < a.only_lo || J >= a.only_hi)) J = -2;
             st.atom = J;
+            st.slot = a.again ? idx : J;
             st.alpha0 = x.split ? item % (4 / NC) * NC : 0;
             st.nent = 0;
             if (J >= 0) {
@@ -1359,7 +1362,11 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
         }
         __syncthreads();
         const int J = st.atom;
-        if (J < 0) break;
+        if (J == -1) break;
+        if (J < 0) {
+            __syncthreads();
+            continue;
+        }
         if (st.n_at > a.na_max) {
             if (threadIdx.x == 0) flag(a.status, DEV_CAPACITY);
             __syncthreads();

@@ -74,6 +74,11 @@ int clear_status(elses_system s, cudaStream_t st) {
     return 0;
 }
 
+// Doubles of a column in the store of bases: U, SU and HU (bvec each), the Gram-Schmidt coefficients, H'.
+static size_t kept_stride(int nm, size_t bvec) {
+    return (3 * bvec + (size_t)nm * nm + (size_t)nm * (nm + 1) / 2 + 3) & ~(size_t)3;
+}
+
 // Column storage, Krylov launch shape and batch buffers for the current sizes.
 int prepare_columns(elses_system s) {
     s->nu_max = nu_of_params(s->p);
@@ -158,7 +163,10 @@ int prepare_columns(elses_system s) {
             int bps_max = (s->p.krylov_block || half) ? bps : krylov_blocks_per_sm_max(na, kdeg);
             int fx = -1, fx_dense = -1;
             const int form = fx_form_for(s->n, s->num_sms);
-            const int fx_b = s->p.krylov_block ? 0 : fx_blocks_per_sm(form, na, s->max_nb + 1, nm, s->p.reorth != 0, s->p.force_mode == 1);
+            // (the class is the fixed-point kernel's only where its form that keeps the bases fits as well: the
+            // exact gradient builds the columns with the kernel that the energy pass used)
+            const auto fx_fit = [&](bool store) { return fx_blocks_per_sm(form, na, s->max_nb + 1, nm, s->p.reorth != 0, store); };
+            const int fx_b = s->p.krylov_block || fx_fit(true) < 1 ? 0 : fx_fit(s->p.force_mode == 1);
             const auto shape = [&](bool fixed, int b, int b_max) {
                 if (s->p.k3_ctas_per_sm > 0) return std::min(b_max, s->p.k3_ctas_per_sm);
                 if (key < (int)s->tuned_bps.size() && s->tuned_bps[key] > 0 && s->tuned_fx[key] == fixed)
@@ -228,7 +236,7 @@ int prepare_columns(elses_system s) {
     s->use_store = false;
     if (s->p.force_mode == 1 && !s->p.two_pass && !s->p.krylov_block) {
         s->bvec = (size_t)nm * s->na_max * 4;
-        s->bstride = (3 * s->bvec + (size_t)nm * nm + (size_t)nm * (nm + 1) / 2 + 3) & ~(size_t)3;
+        s->bstride = kept_stride(nm, s->bvec);
         const size_t need = M * s->bstride;
         if (need * sizeof(double) <= (size_t(48) << 30)) {
             TRY(s->bstore.ensure(need));
@@ -454,6 +462,27 @@ void launch_krylov(elses_system s, const KrylovArgs& ka, int fx, int grid, int b
     else krylov_columns(ka, grid, bps, st);
 }
 
+// The Krylov build of ka.n_items atoms of a size class, with their bases kept where ka.bstore is set. For
+// caller matrices the fixed-point kernel where they suit it, decided on the device, else the FP64 one.
+static void launch_class(elses_system s, KrylovArgs ka, const elses_system_s::K3Launch& L, cudaStream_t st) {
+    const bool store = ka.bstore != nullptr;
+    const int form = !s->user_hs ? L.fx : s->fx_user ? L.fx_dense : -1;
+    ka.na_max = L.na;
+    if (form >= 0) {
+        int bps = fx_blocks_per_sm(form, L.na, s->max_nb + 1, s->nu_max, s->p.reorth != 0, store);
+        if (!s->user_hs) bps = std::min(bps, L.bps);
+        else if (s->p.k3_ctas_per_sm > 0) bps = std::min(bps, s->p.k3_ctas_per_sm);
+        launch_krylov(s, ka, form, std::min(fx_items(form, ka.n_items), s->num_sms * bps), bps, st);
+        s->stats.launches++;
+        if (!s->user_hs) return;
+        ka.skip = &s->fx_scale.p[1].ok;
+    }
+    ka.half = store ? 0 : L.half;                  // half-warp columns do not keep their bases:
+    if (store) ka.na_max = (L.na + 31) / 32 * 32;   // a warp each, with room for whole slots
+    launch_krylov(s, ka, -1, std::min(ka.n_items, L.grid64), L.bps64, st);
+    s->stats.launches++;
+}
+
 // Krylov build + projected eigenproblem for atoms [b, e). Writes V and UP either to the stored
 // arrays or to the batch buffers (two-pass), returning the pointers used. form_v false leaves V
 // unformed; in the stored workflow that holds for a batch of every atom (its factors then stay in
@@ -494,8 +523,6 @@ int run_batch(elses_system s, int b, int e, bool stored, double** V_out, int* v_
     for (size_t i = 0; i < ls.size(); ++i) {
         const auto& L = *ls[i];
         cudaStream_t lst = (conc && i != main_cls) ? s->side : st;
-        ka.na_max = L.na;
-        ka.half = L.half;
         ka.order = s->order.p + L.item_begin;
         ka.n_items = L.item_count;
         ka.scratch = s->kscratch.p + L.scratch_off;
@@ -506,18 +533,7 @@ int run_batch(elses_system s, int b, int e, bool stored, double** V_out, int* v_
             CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int), lst));
             ka.queue = q;
         }
-        if (s->user_hs && s->fx_user && L.fx_dense >= 0) {
-            // the fixed-point kernel where the matrices suit it, decided on the device, else the FP64 one
-            const int fb = fx_blocks_per_sm(L.fx_dense, L.na, s->max_nb + 1, s->nu_max, s->p.reorth != 0, s->p.force_mode == 1);
-            const int bps = s->p.k3_ctas_per_sm > 0 ? std::min(fb, s->p.k3_ctas_per_sm) : fb;
-            launch_krylov(s, ka, L.fx_dense, std::min(fx_items(L.fx_dense, L.item_count), s->num_sms * bps), bps, lst);
-            s->stats.launches++;
-            ka.skip = &s->fx_scale.p[1].ok;
-        }
-        if (s->user_hs) launch_krylov(s, ka, -1, L.grid64, L.bps64, lst);
-        else launch_krylov(s, ka, L.fx, L.grid, L.bps, lst);
-        ka.skip = nullptr;
-        s->stats.launches++;
+        launch_class(s, ka, L, lst);
         s->stats.krylov_launches++;
     }
     if (conc) TRY(join_side(s, st));
@@ -546,32 +562,58 @@ int run_batch(elses_system s, int b, int e, bool stored, double** V_out, int* v_
 }
 
 // Exact dOmega/dH and s_scale * dOmega/dS at mu of the columns of atoms [lo, hi) into gH, gS
-// ([nnzb][16], overwritten): per batch, the adjoint kernel per size class, after the batch's
-// Krylov columns are recomputed when V is not kept (two-pass mode).
+// ([nnzb][16], overwritten): per batch and size class, the adjoint kernel over the bases that the
+// energy pass kept, or else over those of a second build of the class, a few waves of atoms at a time.
 int adjoint_impl(elses_system s, double mu, int lo, int hi, double* gH, double* gS, double s_scale,
                  cudaStream_t st, const double* mu_dev) {
     const int nm = s->nu_max;
     const int kdeg = s->user_hs ? s->max_nb : s->deg_cap;
+    const bool again = !s->use_store;
     TRY(s->adj_acc.ensure(4 * 16 * (size_t)s->nnzb));
     CUDA_TRY(cudaMemsetAsync(s->adj_acc.p, 0, sizeof(unsigned long long) * 4 * 16 * (size_t)s->nnzb, st));
     // launch shapes and scratch: the Krylov kernel's size classes, the adjoint's own residency
     if ((int)s->adj_bps.size() != s->na_max / 32 + 1) s->adj_bps.assign(s->na_max / 32 + 1, 0);
-    size_t need = 0;
-    std::vector<int> grid(s->k3_launches.size(), 0);
-    std::vector<size_t> off(s->k3_launches.size(), 0);
-    for (size_t i = 0, used = 0; i < s->k3_launches.size(); ++i) {
-        const auto& L = s->k3_launches[i];
-        const int na = (L.na + 31) / 32 * 32;   // the adjoint keeps one warp per column
+    const size_t nl = s->k3_launches.size();
+    const auto na_of = [&](size_t i) { return (s->k3_launches[i].na + 31) / 32 * 32; };   // one warp per column
+    const auto bstride_of = [&](int na) { return kept_stride(nm, (size_t)nm * na * 4); };
+    std::vector<int> grid(nl, 0);
+    for (size_t i = 0; i < nl; ++i) {
+        const int na = na_of(i);
         int& bps = s->adj_bps[na / 32];
         if (bps == 0) bps = adjoint_blocks_per_sm(na, kdeg);
         if (bps < 1) return fail(ELSES_ERR_CAPACITY, "adjoint kernel cannot be resident (%d-atom class)", na);
-        grid[i] = std::min(L.item_count, s->num_sms * bps);
-        if (i == 0 || L.batch_begin != s->k3_launches[i - 1].batch_begin) used = 0;
-        off[i] = used;     // the class launches of a batch run at the same time: own scratch each
-        used += (size_t)grid[i] * kWarpsPerAtom * adjoint_warp_doubles(nm, na);
+        grid[i] = std::min(s->k3_launches[i].item_count, s->num_sms * bps);
+    }
+    // the class launches of a batch run at the same time: own scratch and kept bases each
+    std::vector<size_t> off(nl, 0), boff(nl, 0);
+    size_t need = 0;
+    for (size_t i = 0, used = 0; i < nl; ++i) {
+        if (i == 0 || s->k3_launches[i].batch_begin != s->k3_launches[i - 1].batch_begin) used = 0;
+        off[i] = used;
+        used += (size_t)grid[i] * kWarpsPerAtom * adjoint_warp_doubles(nm, na_of(i));
         need = std::max(need, used);
     }
     TRY(s->ascratch.ensure(need));
+    std::vector<int> chunk(nl, 0);
+    if (again) {
+        // atoms built at a time: eight waves of the adjoint kernel, fewer where that takes more than 4 GB
+        // or than there is
+        TRY(s->adj_nu.ensure(s->M));
+        const auto plan = [&](int waves) {
+            size_t most = 0, used = 0;
+            for (size_t i = 0; i < nl; ++i) {
+                if (i == 0 || s->k3_launches[i].batch_begin != s->k3_launches[i - 1].batch_begin) used = 0;
+                chunk[i] = (int)std::min<long long>(s->k3_launches[i].item_count, (long long)waves * grid[i]);
+                boff[i] = used;
+                used += (size_t)chunk[i] * 4 * bstride_of(na_of(i));
+                most = std::max(most, used);
+            }
+            return most;
+        };
+        int waves = 8;
+        while (waves > 1 && (plan(waves) > (size_t(4) << 30) / sizeof(double) || !s->gstore.try_ensure(plan(waves)))) waves /= 2;
+        TRY(s->gstore.ensure(plan(waves)));
+    }
     if (!s->p.two_pass) TRY(ensure_V(s, st));
     for (int b = 0; b < s->n; b += s->batch_atoms) {
         const int e = std::min(s->n, b + s->batch_atoms);
@@ -599,12 +641,12 @@ int adjoint_impl(elses_system s, double mu, int lo, int hi, double* gH, double* 
         ga.scratch = s->ascratch.p;
         ga.atom_lo = lo;
         ga.atom_hi = hi;
-        ga.bstore = s->use_store ? s->bstore.p : nullptr;
-        ga.bstride = s->bstride;
-        ga.bvec = s->bvec;
+        ga.nu_kept = again ? s->adj_nu.p : s->nu_eff.p;
         KrylovArgs ka = krylov_args(s, b, e);
-        ka.flops = nullptr;
         ka.UP = nullptr;
+        ka.again = again;
+        ka.only_lo = lo;
+        ka.only_hi = hi;
         s->tic(T_ADJOINT, st);
         std::vector<size_t> li;
         for (size_t i = 0; i < s->k3_launches.size(); ++i)
@@ -618,17 +660,33 @@ int adjoint_impl(elses_system s, double mu, int lo, int hi, double* gH, double* 
             const size_t i = li[t];
             const auto& L = s->k3_launches[i];
             cudaStream_t lst = (conc && t != main_cls) ? s->side : st;
-            ka.na_max = (L.na + 31) / 32 * 32;
-            ka.half = 0;
-            ka.order = s->order.p + L.item_begin;
-            ka.n_items = L.item_count;
             int* q = s->counters.p + kQueue0 + (int)std::min<size_t>(t, kCounters - kQueue0 - 1);
-            CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int), lst));
-            ka.queue = q;
             AdjointArgs gl = ga;
             gl.scratch = s->ascratch.p + off[i];
-            adjoint_columns(ka, gl, grid[i], lst);
-            s->stats.launches++;
+            const int step = again ? chunk[i] : L.item_count;
+            for (int c0 = 0; c0 < L.item_count; c0 += step) {
+                KrylovArgs kc = ka;
+                kc.order = s->order.p + L.item_begin + c0;
+                kc.n_items = std::min(step, L.item_count - c0);
+                if (again) {
+                    kc.bstore = s->gstore.p + boff[i];
+                    kc.bvec = (size_t)nm * na_of(i) * 4;
+                    kc.bstride = bstride_of(na_of(i));
+                    kc.nu_eff = s->adj_nu.p;
+                    kc.flops = ga.flops;
+                    kc.scratch = s->kscratch.p + L.scratch_off;
+                    CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int), lst));
+                    kc.queue = q;
+                    launch_class(s, kc, L, lst);
+                }
+                kc.na_max = na_of(i);
+                kc.half = 0;
+                kc.nu_eff = s->nu_eff.p;
+                CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int), lst));
+                kc.queue = q;
+                adjoint_columns(kc, gl, std::min(grid[i], kc.n_items), lst);
+                s->stats.launches++;
+            }
         }
         if (conc) TRY(join_side(s, st));
         s->toc(st);

@@ -145,6 +145,8 @@ struct elses_system_s {
     DevBuf<double> ascratch, adjH, adjS;   // exact-gradient scratch and its pattern gradients
     DevBuf<unsigned long long> adj_acc;    // their exact fixed-point sums (AdjointArgs::acc)
     DevBuf<double> bstore;                 // per-column bases kept for the exact gradient
+    DevBuf<double> gstore;                 // or those of the columns it is taking, and their lengths
+    DevBuf<int> adj_nu;
     size_t bstride = 0, bvec = 0;
     bool use_store = false;
     // the eigen-factors of every column are in the batch buffers and the stored V is not formed
