@@ -262,7 +262,9 @@ struct FxState {
     FxLayout v;
     FxScale sc;
     const int4* rec;
-    int4 *gU, *gY, *gX;     // basis vectors in global scratch, `units` apart, and a place for xd
+    int4 *gU, *gY;          // basis vectors in global scratch, `units` apart
+    double2 *gD, *hd;       // lead: the vectors in FP64 (in units of X), `units` apart, and H u_n, then w
+    double2* xa;            // shared memory for the first kLead + 1 of them in turn, or null
     unsigned tmem;
     int n_at, NS, units, upt, qJ, nent, nu, nm, alpha0;
     int kT, kS, kY;         // U[0, kT) in tensor memory, U[kT, kS) and SU[0, kY) in shared memory
@@ -273,7 +275,7 @@ struct FxState {
     unsigned top[2][NC];    // the same of the lead's FP64 vectors: largest high word
     int bH[NC], bS[NC];     // H u_n = f 2^bH P, S u_n = f 2^bS Y
     int sP[NC];             // lead: P = xd 2^sP, rounded
-    double2* xd;            // lead: u_n (in units of X), then H u_n or w, in FP64
+    int lead, small;        // steps of the lead; whether an atom is still too small to leave it
     double Es, Ep;
     double hh[2][NC];       // |P|^2 of the even and the odd steps
     int q[NC], done[NC], nue[NC], we[NC], big[NC];
@@ -317,6 +319,7 @@ __device__ __forceinline__ void fx_max(unsigned m, unsigned* to) {
     for (int o = NC; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) < NC) atomicMax(to, m);
 }
+__device__ __forceinline__ bool fx_zero(const double2 v) { return v.x == 0.0 && v.y == 0.0; }
 __device__ __forceinline__ unsigned fx_top(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 // s with 2^55 <= 2^s v < 2^56 for the largest v, of high word `top`
 __device__ __forceinline__ int fx_lead_shift(unsigned top) { return top ? 55 - ((int)(top >> 20) - 1023) : 0; }
@@ -374,7 +377,7 @@ __device__ __forceinline__ int2 fx_hi(const int4& v) { return make_int2(v.z, v.w
 // 6e-12); a state of weight 1e-5 at the rim of a graphite cluster 3e-9, 1.5e-9, 2e-10, 2e-10. Density
 // matrices are on a par with FP64's from five on. Six steps: each costs 3% of the kernel (4096 atoms: 28
 // ms without, 29.8 with 3, 32.8 with 6, 34.9 with 8).
-constexpr int kLead = 6;
+constexpr int kLead = 6, kSmall = 10;
 
 template <int T, int kMinB>
 struct FxTmem {
@@ -646,14 +649,15 @@ __device__ __forceinline__ void fx_products_dense(FxState<NC>& st) {
     fx_or<NC>(mS, &st.bits[1][tc]);
 }
 
-// The lead's form of fx_products: FP64 products of xd into P and Y (as FP64), entries whose neighbour
-// is not reached yet left out.
+// The lead's form of fx_products: FP64 products of u_n into P and Y (as FP64), entries whose neighbour
+// is not reached yet left out. An atom that is reached now keeps the lead going: there may be more behind it.
 template <int NC, int T, bool kDense>
-__device__ __forceinline__ void fx_products_lead(const KrylovArgs& a, FxState<NC>& st) {
+__device__ __forceinline__ void fx_products_lead(const KrylovArgs& a, FxState<NC>& st, int n) {
     constexpr int G = T / NC;
     const int tid = threadIdx.x, tc = tid % NC, g = tid / NC, NS = st.NS;
     const short* row_at = fx_at<short>(st.v.row_at);
-    const char* xc = reinterpret_cast<const char*>(st.xd + tc);
+    const double2* xd = n <= kLead && st.xa ? st.xa : st.gD + (size_t)n * st.units;
+    const char* xc = reinterpret_cast<const char*>(xd + tc);
     double2 *PH = fx_at<double2>(st.v.P), *PS = fx_at<double2>(st.v.Y);
     unsigned mH = 0, mS = 0;
 #pragma unroll 1
@@ -664,10 +668,11 @@ __device__ __forceinline__ void fx_products_lead(const KrylovArgs& a, FxState<NC
         const size_t b0 = (size_t)fx_at<int>(st.v.base)[q];
         const char* rb = reinterpret_cast<const char*>(a.skr + 12 * b0);
         const int d = fx_at<int>(st.v.deg)[q], u01 = fx_unit<NC>(q, 0, tc), u23 = fx_unit<NC>(q, 1, tc);
+        const double2 x01 = xd[u01], x23 = xd[u23];
         double2 s01 = make_double2(0.0, 0.0), s23 = s01;
         if (!kDense) {
-            s01 = st.xd[u01];
-            s23 = st.xd[u23];
+            s01 = x01;
+            s23 = x23;
         }
         double2 h01 = make_double2(st.Es * s01.x, st.Ep * s01.y), h23 = make_double2(st.Ep * s23.x, st.Ep * s23.y);
 #pragma unroll 1
@@ -675,7 +680,7 @@ __device__ __forceinline__ void fx_products_lead(const KrylovArgs& a, FxState<NC
             const unsigned en = ent[k], at = en >> 16;
             const double2 x01 = *reinterpret_cast<const double2*>(xc + at);
             const double2 x23 = *reinterpret_cast<const double2*>(xc + (at ^ (16u * NC)));
-            if (x01.x == 0.0 && x01.y == 0.0 && x23.x == 0.0 && x23.y == 0.0) continue;
+            if (fx_zero(x01) && fx_zero(x23)) continue;
             if (kDense) {
                 const size_t e = 16 * (b0 + (en & 0xffffu) / 256);
                 auto row = [&](const double* X, int r, double y) {
@@ -703,6 +708,7 @@ __device__ __forceinline__ void fx_products_lead(const KrylovArgs& a, FxState<NC
             s23.x = fma(as, u.y, fma(b23.x, x23.x, s23.x));
             s23.y = fma(as, uz.x, fma(b23.x, x23.y, s23.y));
         }
+        if (n + 1 >= kLead && fx_zero(x01) && fx_zero(x23) && !(fx_zero(h01) && fx_zero(h23))) st.small = 1;
         mH = max(max(mH, max(fx_top(h01.x), fx_top(h01.y))), max(fx_top(h23.x), fx_top(h23.y)));
         mS = max(max(mS, max(fx_top(s01.x), fx_top(s01.y))), max(fx_top(s23.x), fx_top(s23.y)));
         PH[u01] = h01;
@@ -881,6 +887,20 @@ __device__ __forceinline__ int fx_norm_test(const KrylovArgs& a, const FxState<N
     return w2 < -bound ? 2 : w2 > bound ? 0 : 1;
 }
 
+// The coefficients of column c for the update: integers, or in the lead FP64 in the place of h.
+template <int NC>
+__device__ __forceinline__ void fx_give_coefs(FxState<NC>& st, int n, int c, const double (&gk)[2]) {
+    const int lane = threadIdx.x & 31;
+    if (n >= st.lead) {
+        fx_coefs(gk, n, fx_at<int2>(st.v.g) + c * st.nm, &st.q[c]);
+        return;
+    }
+    __syncwarp();   // every lane has read h
+    double* g = fx_at<double>(st.v.h) + c * st.nm;
+    if (lane <= n) g[lane] = gk[0];
+    if (lane + 32 <= n) g[lane + 32] = gk[1];
+}
+
 // First warp: S', the coefficients of the update, and the end of the column.
 template <int NC>
 __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st, int n, int c) {
@@ -964,7 +984,7 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
                 }
                 gk[r] = f[k] * (h[k] - eh);
             }
-            fx_coefs(gk, n, fx_at<int2>(st.v.g) + c * nm, &st.q[c]);
+            fx_give_coefs(st, n, c, gk);
         }
     }
 }
@@ -998,7 +1018,7 @@ __device__ __forceinline__ void fx_scalars_h(const KrylovArgs& a, FxState<NC>& s
 
 // w = P - sum_{k <= n} g_k X_k as 64-bit numbers, into X or in place (into P).
 template <int NC, int T, int kMinB>
-__device__ __forceinline__ void fx_update(FxState<NC>& st, int n, bool into_x, unsigned long long* bits, unsigned* top) {
+__device__ __forceinline__ void fx_update(FxState<NC>& st, int n, bool into_x, unsigned long long* bits) {
     const int tid = threadIdx.x, tc = tid % NC, units = st.units, upt = st.upt, kT = st.kT, kS = st.kS;
     const unsigned tm = FxTmem<T, kMinB>::base(st.tmem);
     const int4* P = fx_at<int4>(st.v.P);
@@ -1006,7 +1026,6 @@ __device__ __forceinline__ void fx_update(FxState<NC>& st, int n, bool into_x, u
     const int2* g = fx_at<int2>(st.v.g) + tc * st.nm;
     const int q = st.q[tc];
     unsigned long long mW = 0;
-    unsigned mT = 0;
 #pragma unroll 1
     for (int i0 = 0; i0 < upt; i0 += 2) {
         Fx acc[4];
@@ -1055,33 +1074,47 @@ __device__ __forceinline__ void fx_update(FxState<NC>& st, int n, bool into_x, u
         for (int i = 0; i < 2; ++i) {
             const int u = tid + (i0 + i) * T;
             if (i0 + i < upt && u < units) {
-                if (n < kLead) {
-                    const double2 h = st.xd[u];
-                    const double fh = fx_pow2(st.sP[tc]), fg = fx_pow2(q);
-                    double2 w;
-                    w.x = fma(h.x, fh, -((double)fx_fold(acc[2 * i]) * fg));
-                    w.y = fma(h.y, fh, -((double)fx_fold(acc[2 * i + 1]) * fg));
-                    mT = max(mT, max(fx_top(w.x), fx_top(w.y)));
-                    reinterpret_cast<double2*>(W)[u] = w;
-                } else {
-                    const int4 p = P[u];
-                    longlong2 w;
-                    w.x = fx_shr(((long long)p.x << 28) + p.y, q) - fx_fold(acc[2 * i]);
-                    w.y = fx_shr(((long long)p.z << 28) + p.w, q) - fx_fold(acc[2 * i + 1]);
-                    mW |= fx_abs_bits(w.x) | fx_abs_bits(w.y);
-                    W[u] = w;
-                }
+                const int4 p = P[u];
+                longlong2 w;
+                w.x = fx_shr(((long long)p.x << 28) + p.y, q) - fx_fold(acc[2 * i]);
+                w.y = fx_shr(((long long)p.z << 28) + p.w, q) - fx_fold(acc[2 * i + 1]);
+                mW |= fx_abs_bits(w.x) | fx_abs_bits(w.y);
+                W[u] = w;
             }
         }
         __syncwarp();
     }
-    if (st.done[tc]) {
-        mW = 0;
-        mT = 0;
-    }
+    if (st.done[tc]) mW = 0;
     __syncwarp();
-    if (n < kLead) fx_max<NC>(mT, top + tc);
-    else fx_or<NC>(mW, bits + tc);
+    fx_or<NC>(mW, bits + tc);
+}
+
+// The same in the lead, in FP64: w = 2^sP h - sum_{k <= n} g_k u_k, h and u_k as FP64.
+template <int NC, int T>
+__device__ __forceinline__ void fx_update_lead(FxState<NC>& st, int n, bool into_x, unsigned* top) {
+    const int tid = threadIdx.x, tc = tid % NC, units = st.units;
+    double2* W = fx_at<double2>(into_x ? st.v.X : st.v.P);
+    const double* g = fx_at<double>(st.v.h) + tc * st.nm;
+    const double fh = fx_pow2(st.sP[tc]);
+    unsigned mT = 0;
+#pragma unroll 1
+    for (int u = tid; u < units; u += T) {
+        double2 w = st.hd[u];
+        w.x *= fh;
+        w.y *= fh;
+        const double2* q = st.gD + u;
+#pragma unroll 4
+        for (int k = 0; k <= n; ++k, q += units) {
+            const double2 v = *q;
+            w.x = fma(-g[k], v.x, w.x);
+            w.y = fma(-g[k], v.y, w.y);
+        }
+        mT = max(mT, max(fx_top(w.x), fx_top(w.y)));
+        W[u] = w;
+    }
+    if (st.done[tc]) mT = 0;
+    __syncwarp();
+    fx_max<NC>(mT, top + tc);
 }
 
 // Where vector k of U lives outside tensor memory.
@@ -1097,7 +1130,8 @@ __device__ __forceinline__ void fx_start(FxState<NC>& st) {
     int4* X = fx_at<int4>(st.v.X);
     for (int u = tid; u < units; u += T) {
         X[u] = make_int4(0, 0, 0, 0);
-        st.xd[u] = make_double2(0.0, 0.0);
+        st.gD[u] = make_double2(0.0, 0.0);
+        if (st.xa) st.xa[u] = make_double2(0.0, 0.0);
     }
     for (int q = tid; q < red_words; q += T) fx_at<int>(st.v.red)[q] = 0;
     if (tid < NC) {
@@ -1106,13 +1140,17 @@ __device__ __forceinline__ void fx_start(FxState<NC>& st) {
         st.done[tid] = st.big[tid] = st.q[tid] = 0;
         st.nue[tid] = st.nu;
     }
-    if (tid == 0) st.live = NC;
+    if (tid == 0) {
+        st.live = NC;
+        st.lead = kLead;
+        st.small = 0;
+    }
     __syncthreads();
     if (tid < NC) {
-        const int al = st.alpha0 + tid;
-        int* w = reinterpret_cast<int*>(X + fx_unit<NC>(st.qJ, al >> 1, tid));
-        w[2 * (al & 1)] = 1 << 28;
-        reinterpret_cast<double*>(st.xd + fx_unit<NC>(st.qJ, al >> 1, tid))[al & 1] = 0x1p56;
+        const int al = st.alpha0 + tid, at = fx_unit<NC>(st.qJ, al >> 1, tid);
+        reinterpret_cast<int*>(X + at)[2 * (al & 1)] = 1 << 28;
+        reinterpret_cast<double*>(st.gD + at)[al & 1] = 0x1p56;
+        if (st.xa) reinterpret_cast<double*>(st.xa + at)[al & 1] = 0x1p56;
     }
     __syncthreads();
     const unsigned tm = FxTmem<T, kMinB>::base(st.tmem);
@@ -1130,12 +1168,12 @@ __device__ __forceinline__ void fx_take_products(FxState<NC>& st, int n) {
     const int tid = threadIdx.x, tc = tid % NC, units = st.units;
     int4 *P = fx_at<int4>(st.v.P), *Y = fx_at<int4>(st.v.Y);
     int4* yn = n < st.kY ? fx_at<int4>(st.v.cache) + (st.kS - st.kT + n) * units : st.gY + (size_t)n * units;
-    if (n < kLead) {
+    if (n < st.lead) {
         const int sH = fx_lead_shift(st.top[0][tc]), sS = fx_lead_shift(st.top[1][tc]);
         const double fH = fx_pow2(sH), fS = fx_pow2(sS);
         for (int u = tid; u < units; u += T) {
             const double2 h = reinterpret_cast<const double2*>(P)[u];
-            st.xd[u] = h;
+            st.hd[u] = h;
             P[u] = fx_lead_split(h, fH);
             const int4 y = fx_lead_split(reinterpret_cast<const double2*>(Y)[u], fS);
             Y[u] = y;
@@ -1163,33 +1201,49 @@ __device__ __forceinline__ void fx_take_products(FxState<NC>& st, int n) {
 }
 
 // w (64-bit numbers in X; FP64 in the lead, sh then the power of two it is multiplied by) becomes
-// X_(n+1), in X and in the basis.
+// X_(n+1), in X and in the basis. The lead goes on while an atom that is reached stays below 2^-kSmall of
+// the largest in the last two vectors.
 template <int NC, int T, int kMinB>
 __device__ __forceinline__ void fx_take_vector(FxState<NC>& st, int n, int sh) {
     const int tid = threadIdx.x, units = st.units, upt = st.upt;
-    const bool dead = st.done[tid % NC] != 0;
+    const bool dead = st.done[tid % NC] != 0, in_lead = n < st.lead;
     int4* X = fx_at<int4>(st.v.X);
     const double lead = fx_pow2(sh);
     const unsigned tm = FxTmem<T, kMinB>::base(st.tmem);
+    double2* const D = st.gD + (size_t)n * units;
+    bool small = false;
     for (int i = 0; i < upt; ++i) {
         const int u = tid + i * T;
         int4 w = make_int4(0, 0, 0, 0);
-        if (u < units) {
-            if (n < kLead) {
+        if (in_lead) {
+            unsigned top = 0;
+            if (u < units) {
                 double2 wd = make_double2(0.0, 0.0);
                 if (!dead) wd = reinterpret_cast<const double2*>(X)[u];
                 wd.x *= lead;
                 wd.y *= lead;
-                st.xd[u] = wd;
+                if (n + 1 >= kLead) {
+                    const double2 before = D[u];
+                    top = max(max(fx_top(wd.x), fx_top(wd.y)), max(fx_top(before.x), fx_top(before.y)));
+                }
+                D[units + u] = wd;
+                if (st.xa && n + 1 <= kLead) st.xa[u] = wd;
                 w = fx_lead_split(wd, 1.0);
-            } else if (!dead) {
-                w = fx_norm2(reinterpret_cast<const longlong2*>(X)[u], sh);
+                X[u] = w;
             }
+            __syncwarp();
+            if (n + 1 >= kLead) {   // an atom's other two orbitals are NC lanes on
+                top = max(top, __shfl_xor_sync(0xffffffffu, top, NC));
+                small |= !dead && top > 0u && top < (unsigned)(1023 + 56 - kSmall) << 20;
+            }
+        } else if (u < units) {
+            if (!dead) w = fx_norm2(reinterpret_cast<const longlong2*>(X)[u], sh);
             X[u] = w;
         }
         if (n + 1 < st.kT) fx_tmem_st(tm + 4 * ((n + 1) * upt + i), w);
         else if (u < units) fx_ubase(st, n + 1)[u] = w;
     }
+    if (small) st.small = 1;
 }
 
 // The second classical pass between its two updates: w (64-bit numbers in P) into split form, its
@@ -1199,11 +1253,11 @@ __device__ __forceinline__ void fx_second_coefs(FxState<NC>& st, int n, int sh) 
     const int tid = threadIdx.x, c = tid >> 5, lane = tid & 31, nm = st.nm, RC = 3 * nm + 1, RS = NC * RC;
     int4* P = fx_at<int4>(st.v.P);
     int* red = fx_at<int>(st.v.red);
-    if (n < kLead) {
+    if (n < st.lead) {
         const double lead = fx_pow2(sh);
         for (int u = tid; u < st.units; u += T) {
             const double2 wd = reinterpret_cast<const double2*>(P)[u];
-            st.xd[u] = wd;
+            st.hd[u] = wd;
             P[u] = fx_lead_split(wd, lead);
         }
         if (tid < NC) st.sP[tid] = sh;
@@ -1220,7 +1274,7 @@ __device__ __forceinline__ void fx_second_coefs(FxState<NC>& st, int n, int sh) 
             if (k <= n)
                 gk[r] = fx_at<double>(st.v.f)[c * nm + k] * (fx_at<double>(st.v.s)[c * nm + k] * fx_red_get(red + c * RC + k, RS));
         }
-        fx_coefs(gk, n, fx_at<int2>(st.v.g) + c * nm, &st.q[c]);
+        fx_give_coefs(st, n, c, gk);
     }
     __syncthreads();
     for (int q = tid; q < 3 * RS; q += T) red[q] = 0;
@@ -1322,9 +1376,10 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
         st.v = fx_layout<NC, T>(a.na_max, a.nu_max, a.deg_max + 1, a.reorth != 0, a.bstore != nullptr);
         st.sc = *x.scale;
         st.rec = x.rec;
-        st.gU = reinterpret_cast<int4*>(a.scratch) + (2 * cta_units + (size_t)a.na_max * 2 * NC) * blockIdx.x;
+        st.gU = reinterpret_cast<int4*>(a.scratch) + (3 * cta_units + (size_t)a.na_max * 2 * NC) * blockIdx.x;
         st.gY = st.gU + cta_units;
-        st.gX = st.gY + cta_units;
+        st.gD = reinterpret_cast<double2*>(st.gY + cta_units);
+        st.hd = st.gD + cta_units;
         st.Es = x.Es;
         st.Ep = x.Ep;
         st.nm = a.nu_max;
@@ -1355,9 +1410,9 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
                 st.kT = min((Tm::units - 1) / upt, nu) & ~3;
                 st.kS = st.kT + min(nu - st.kT, vecs);
                 st.kY = min(nu, vecs - (st.kS - st.kT));
-                // xd: the last vector's place in shared memory while that is free, else scratch
-                st.xd = reinterpret_cast<double2*>(st.kS > st.kT && st.kS - 1 > kLead
-                                                       ? fx_at<int4>(st.v.cache) + (st.kS - 1 - st.kT) * units : st.gX);
+                // the last vector's place in shared memory while that is free
+                st.xa = st.kS > st.kT && st.kS - 1 > kLead
+                            ? reinterpret_cast<double2*>(fx_at<int4>(st.v.cache) + (st.kS - 1 - st.kT) * units) : nullptr;
             }
         }
         __syncthreads();
@@ -1380,7 +1435,8 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
             fx_start<NC, T, kMinB>(st);
             const int nu = st.nu;
             for (int n = 0; n < nu; ++n) {
-                if (n < kLead) fx_products_lead<NC, T, kDense>(a, st);
+                const bool lead = n < st.lead;
+                if (lead) fx_products_lead<NC, T, kDense>(a, st, n);
                 else if constexpr (kDense) fx_products_dense<NC, T>(st);
                 else fx_products<NC, T>(st);
                 __syncthreads();
@@ -1409,11 +1465,12 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
                     break;
                 }
                 for (int pass = st.overlap ? 1 : 0; pass < 2; ++pass) {
-                    fx_update<NC, T, kMinB>(st, n, pass == 1, st.bits[pass], st.top[pass]);
+                    if (lead) fx_update_lead<NC, T>(st, n, pass == 1, st.top[pass]);
+                    else fx_update<NC, T, kMinB>(st, n, pass == 1, st.bits[pass]);
                     __syncthreads();
                     const int tc = threadIdx.x % NC;
-                    const int sh = n < kLead ? fx_lead_shift(st.top[pass][tc]) : fx_shift(st.bits[pass][tc]);
-                    if (threadIdx.x < NC) st.we[tc] += n < kLead ? -sh : st.q[tc] + sh;   // P = 2^we (the new integers)
+                    const int sh = lead ? fx_lead_shift(st.top[pass][tc]) : fx_shift(st.bits[pass][tc]);
+                    if (threadIdx.x < NC) st.we[tc] += lead ? -sh : st.q[tc] + sh;   // P = 2^we (the new integers)
                     if (pass == 1) fx_take_vector<NC, T, kMinB>(st, n, sh);
                     else fx_second_coefs<NC, T>(st, n, sh);
                 }
@@ -1421,6 +1478,10 @@ __global__ void __launch_bounds__(T, kMinB) k_krylov_fixed(const __grid_constant
                 if (threadIdx.x < NC) {
                     st.bits[0][threadIdx.x] = st.bits[1][threadIdx.x] = 0;
                     st.top[0][threadIdx.x] = st.top[1][threadIdx.x] = 0;
+                }
+                if (threadIdx.x == 0) {
+                    if (st.small) st.lead = max(st.lead, n + 2);
+                    st.small = 0;
                 }
                 __syncthreads();
             }
@@ -1478,7 +1539,7 @@ int fx_blocks_per_sm(int form, int na, int max_row, int nu, bool overlap, bool s
 
 int fx_items(int form, int count) { return count * (4 / kForms[form].nc); }
 
-size_t fx_scratch_doubles(int form, int nu, int na) { return ((size_t)2 * nu + 1) * na * 4 * kForms[form].nc; }
+size_t fx_scratch_doubles(int form, int nu, int na) { return ((size_t)3 * nu + 1) * na * 4 * kForms[form].nc; }
 
 void fx_columns(const KrylovArgs& a, FxArgs x, int form, int grid, int ctas_per_sm, cudaStream_t st) {
     const FxForm& f = kForms[form];
