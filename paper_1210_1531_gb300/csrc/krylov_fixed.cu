@@ -15,7 +15,8 @@
 // (2^-57 of the largest product; FP64 rounds every partial sum), and a vector is rounded to
 // 2^-57 of its largest entry (FP64: each entry to 2^-53 of itself). Sums of integers
 // do not depend on their order, so results are the same for every launch shape. Scalars
-// (norms, H', S', Gram-Schmidt coefficients) are FP64.
+// (norms, H', S', Gram-Schmidt coefficients) are FP64, and so are the vectors of the first steps (the lead,
+// at kLead).
 //
 // Coefficients of the two-centre blocks carry one power-of-two scale per matrix (FxScale): the
 // largest is below 2^57 and the sum of any row's bounds below 2^62 (2^60 for rows of 33 to 64
@@ -368,15 +369,19 @@ __device__ __forceinline__ double fx_red_get(const int* r, int stride) {
 __device__ __forceinline__ int2 fx_lo(const int4& v) { return make_int2(v.x, v.y); }
 __device__ __forceinline__ int2 fx_hi(const int4& v) { return make_int2(v.z, v.w); }
 
-// The first steps (n < kLead) form the products and the new vector in FP64 beside the integers. A step
-// reaches the next shell of the cluster with amplitudes far below the vector's largest (2^-18
-// two bonds on), which FP64 holds to 53 bits of themselves and the integers only to 2^-57 of the
-// largest; where the cluster has a high, localised state there, the later steps amplify what was
-// lost. Poles of such columns against an 80-bit recursion, in eV, with 3, 5, 6 and 8 steps in FP64:
-// a 65 eV state of a close pair in disordered carbon 2e-10, 1e-11, 7e-12, 1e-11 (FP64 throughout
-// 6e-12); a state of weight 1e-5 at the rim of a graphite cluster 3e-9, 1.5e-9, 2e-10, 2e-10. Density
-// matrices are on a par with FP64's from five on. Six steps: each costs 3% of the kernel (4096 atoms: 28
-// ms without, 29.8 with 3, 32.8 with 6, 34.9 with 8).
+// The lead: first steps whose vectors are formed and kept in FP64 beside the integers, which then serve the
+// dot products only. A step reaches the next shell of the cluster with amplitudes far below the vector's
+// largest (2^-18 two bonds on; 2^-20 to 2^-70 behind a bond near the cutoff), which FP64 holds to 53
+// bits of themselves and the integers only to 2^-57 of the largest; where the cluster has a state
+// there, the later steps amplify what was lost. So the lead lasts kLead steps, and on while one of the CTA's
+// columns still reaches new atoms or has an atom below 2^-kSmall of the largest in its last two vectors.
+// Largest pole errors against an 80-bit recursion, in eV, of the 28 to 70 columns where the kernels
+// differ most, FP64 kernel first: graphite with diamond grains (32768 atoms) 2.6e-10 / 2.6e-10, dense
+// disordered carbon (4096) 1.2e-10 / 1.0e-10, diamond (4096) 5.6e-11 / 5.7e-11. (With six steps whatever
+// the amplitudes, and their vectors subtracted as integers, the first was 1.2e-9 and rho there off by 6e-12.)
+// Each step costs 3% of the kernel. kLead 6 and kSmall 10, in ms: diamond 33.2 (32.9 with six steps
+// always), disordered carbon (65536) 303 (298), graphite with grains 184 (156): a third of its atoms have
+// neighbours behind weak bonds. kSmall 12: 177 there, but poles off by 3.0e-10; kSmall 8: 193, 34.3 and 314.
 constexpr int kLead = 6, kSmall = 10;
 
 template <int T, int kMinB>

@@ -18,7 +18,11 @@
 //                  19456 columns, so the time is their number: the update by way of p = s t (Bowdler,
 //                  Martin, Reinsch and Wilkinson's form) instead of D and E each from c^2, s^2 and
 //                  c s, and tests for small entries on the exponents as integers, take 20 a rotation
-//                  instead of 32: 1.72 -> 1.20 ms (256 columns, nu 30), 1.85 -> 1.32 ms (16384).
+//                  instead of 32. That update takes c^2 + s^2 for 1, and 5 more instructions make it
+//                  so to the last bit; without them G(z) was 1.4 times as far off as with the 32 (a
+//                  rotation that is not quite one is at least the same in T and in the vectors there),
+//                  with them 0.97 times, rho 0.85 and rho_E 0.6 times. 1.72 -> 1.36 ms (256 columns,
+//                  nu 30; 1.20 with 20), 1.85 -> 1.50 ms (16384; 1.32).
 //   k_eig_spectra  one thread per (column, vector): the rotations replayed on y give
 //                  c, d, g = Q^T z.
 //   k_eig_vectors  one warp per column, only where V itself is needed (G(z), the adjoint, or
@@ -408,6 +412,10 @@ __global__ void __launch_bounds__(kChaseThreads) k_eig_chase(const EigArgs a) {
                 cr = x * ir;
                 sr = z * ir;
                 r = rr * ir;
+                // c^2 + s^2 = 1, on which the update below relies, to the last bit
+                const double off = -0.5 * fma(cr, cr, fma(sr, sr, -1.0));
+                cr = fma(cr, off, cr);
+                sr = fma(sr, off, sr);
             }
             if (k > lo) E[k - 1] = r;
             const double g = D[k] - p;
