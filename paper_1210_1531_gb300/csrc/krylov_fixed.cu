@@ -950,7 +950,7 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
                 E[pk0 + k] = e;
                 fx_at<float>(st.v.Ef)[(size_t)c * PK + pk0 + k] = (float)e;
                 fx_at<float>(st.v.hf)[c * nm + k] = (float)hk;
-                big |= (__double2hiint(e) & 0x7fffffff) >= (1023 - 30) << 20;
+                big |= (__double2hiint(e) & 0x7fffffff) >= (1023 - 40) << 20;
             }
         }
         if (__any_sync(0xffffffffu, big) && lane == 0) st.big[c] = 1;
@@ -970,8 +970,8 @@ __device__ __forceinline__ void fx_scalars(const KrylovArgs& a, FxState<NC>& st,
                 if (k > n) continue;
                 double eh = 0.0;
                 if (overlap && !st.big[c]) {
-                    // entries of E below 2^-30: their product with h in single precision
-                    // is within 2^-52 of h
+                    // entries of E below 2^-40 (Gram-Schmidt leaves 2^-48 or so): their product with h
+                    // in single precision is within 64 x 2^-64 of h, far below the rounding of h itself
                     const float *Ef = fx_at<float>(st.v.Ef) + (size_t)c * PK, *hf = fx_at<float>(st.v.hf) + c * nm;
                     float e = 0.0f;
                     int at = k * (k + 1) / 2;          // row k up to the diagonal, then column k

@@ -9,7 +9,7 @@
 // GB300 form. On this part the FP64 pipe charges a whole warp instruction whatever the number
 // of active lanes, so every FP64 instruction must carry work on all lanes:
 //   k_eig_reduce   one warp per column, matrices in shared memory: Cholesky (or, where S' = I to
-//                  2^-32, its first-order form), the reduction A = L^-1 H' L^-T and the Householder reduction of A to tridiagonal form T
+//                  2^-40, its first-order form), the reduction A = L^-1 H' L^-T and the Householder reduction of A to tridiagonal form T
 //                  (lanes over rows / columns); the three vectors z = L^-1 (U, SU, HU)_j are
 //                  reflected along, y = Q_H^T z.
 //   k_eig_chase    one thread per column: implicit-shift QR sweeps on T (Wilkinson shift, Givens
@@ -160,9 +160,10 @@ __device__ __forceinline__ bool reduce_cholesky(double* A, double* L, double* in
     return true;
 }
 
-// The same for S' = I + E with |E| < 2^-32, as Gram-Schmidt leaves it: L = I + T with T the strict lower
-// triangle of E and half its diagonal, L^-1 = I - T, up to products of E that are below 2^-64. What T
-// changes in H' and z is below 2^-32 of them, so FP32 sums carry it to 2^-56, without an FP64
+// The same for S' = I + E with |E| < 2^-40, as Gram-Schmidt leaves it (2^-48 or so): L = I + T with T the
+// strict lower triangle of E and half its diagonal, L^-1 = I - T, up to products of E that are below
+// 2^-80. What T changes in H' and z is below 2^-40 of them, so FP32 sums of up to 64 terms carry it to
+// 2^-58 of the largest, 32 times below the rounding of the FP64 triangular solves, without an FP64
 // instruction: the kernel at 16384 columns and nu 30 takes 3.29 ms in the general form and 2.05 ms in
 // this one (0.1 ms of it from the Householder norm by one reciprocal square root). Nothing reads the
 // upper triangles after this: they hold T and H' in FP32 meanwhile.
@@ -231,14 +232,14 @@ __global__ void __launch_bounds__(64) k_eig_reduce(const EigArgs a) {
     const double* Hp = a.Hp + (size_t)c * PK;
     const double* Sp = a.Sp + (size_t)c * PK;
 
-    bool unit = true;      // S' = I to 2^-32
+    bool unit = true;      // S' = I to 2^-40
     unsigned top[4] = {0u, 0u, 0u, 0u};   // upper words of the largest |H'|, |U_j|, |SU_j| and |HU_j|
     for (int q = lane; q < nu * nu; q += 32) {
         const int i = q / nu, k = q % nu;
         const double s = packed(Sp, i, k), h = packed(Hp, i, k);
         A[i * ld + k] = h;
         L[i * ld + k] = s;
-        unit = unit && fabs(i == k ? s - 1.0 : s) < 0x1p-32;
+        unit = unit && fabs(i == k ? s - 1.0 : s) < 0x1p-40;
         top[0] = max(top[0], (unsigned)__double2hiint(h) & 0x7fffffffu);
     }
     for (int k = lane; k < nu; k += 32) {
