@@ -21,9 +21,10 @@
 // Coefficients of the two-centre blocks carry one power-of-two scale per matrix (FxScale): the
 // largest is below 2^57 and the sum of any row's bounds below 2^62 (2^60 for rows of 33 to 64
 // blocks, whose cross terms add up further), so no sum of a sparse product overflows. This form is
-// used only where every row sum lies within 2^8 of the largest, so that each row keeps at least
-// the relative precision FP64 gives it. A caller's dense blocks are held alike, by exact row sums, up
-// to 32 blocks a row: four products a row and block.
+// used only where every row sum lies within 2^5 of the largest, so that a row's coefficients keep 52 bits
+// of its largest at least (one of FP64's 53), and those of rows within 2^4 as many as FP64 gives. Here the
+// row sums of H differ by up to 14 (graphite with grains), of S by up to 5. A caller's dense blocks
+// are held alike, by exact row sums, up to 32 blocks a row: four products a row and block.
 //
 // The host reads whether the form suits a Slater-Koster system when it is built. elses_set_hs does not
 // wait for the device, so with a caller's matrices both kernels are launched and the device decides:
@@ -100,7 +101,7 @@ __global__ void k_fx_scale(const unsigned long long* b, double Es, double Ep, in
     FxScale s{};
     s.ok = max_row <= (dense ? 32 : 64);
     for (int m = 0; m < 2; ++m)
-        if (!(v[m] > 1e-100 && v[m] < 1e100 && v[m] <= 256.0 * lo[m] && v[2 + m] > 0.0)) s.ok = 0;
+        if (!(v[m] > 1e-100 && v[m] < 1e100 && v[m] <= 32.0 * lo[m] && v[2 + m] > 0.0)) s.ok = 0;
     // the second Gram-Schmidt pass takes its coefficients, of order 2^63 sqrt(S), to single precision
     if (!(v[1] > 0x1p-60 && v[1] < 0x1p60)) s.ok = 0;
     if (s.ok) {
