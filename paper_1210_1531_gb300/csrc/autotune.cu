@@ -24,6 +24,11 @@ int autotune_impl(elses_system s, cudaStream_t st) {
     s->tuned_order.assign(s->na_max / 16 + 1, 0);
     s->tuned_half.assign(s->na_max / 16 + 1, 0);
     const bool half_ok = s->p.k3_lanes != 32 && s->p.force_mode == 0 && !s->p.krylov_block;
+    // whether a class of na atoms is the fixed-point kernel's, which has no half-warp form
+    const auto fx_takes = [&](int na) {
+        return !s->user_hs && s->fx && s->fx_room(false) &&
+               fx_blocks_per_sm(fx_form_for(s->n, s->num_sms), na, s->max_nb + 1, nm, s->p.reorth != 0, true) > 0;
+    };
     // odd classes (an odd number of 16-atom slots) that the occupancy heuristic merged into the
     // next even class are planned on their own for the comparison below, so that half-warp and
     // whole-warp columns are timed for every odd class that has atoms
@@ -31,7 +36,7 @@ int autotune_impl(elses_system s, cudaStream_t st) {
         bool split = false;
         for (int a = 0; a < s->n; ++a) {
             const int k = (s->h_clsize[a] + 15) / 16;
-            if ((k & 1) && k < (int)s->tuned_half.size() && !s->tuned_half[k] && !s->fx) {
+            if ((k & 1) && k < (int)s->tuned_half.size() && !s->tuned_half[k] && !fx_takes(16 * k)) {
                 s->tuned_half[k] = 1;
                 split = true;
             }
