@@ -14,7 +14,8 @@
 // a dot product has no rounding but that of the dropped terms and one rounding per partial sum
 // (2^-57 of the largest product; FP64 rounds every partial sum), and a vector is rounded to
 // 2^-57 of its largest entry (FP64: each entry to 2^-53 of itself). Sums of integers
-// do not depend on their order, so results are the same for every launch shape. Scalars
+// do not depend on their order: a form's results are the same for every grid, queue and batch (the two
+// forms, fx_form_for, cut their partial sums differently). Scalars
 // (norms, H', S', Gram-Schmidt coefficients) are FP64, and so are the vectors of the first steps (the lead,
 // at kLead).
 //
@@ -388,7 +389,7 @@ constexpr int kLead = 6, kSmall = 10;
 template <int T, int kMinB>
 struct FxTmem {
     // whole groups of four warps share the columns, and an allocation is a power of two
-    static_assert(T % 128 == 0 && (kMinB == 1 || kMinB == 2 || kMinB == 4), "tensor memory split");
+    static_assert(T % 128 == 0 && (kMinB == 1 || kMinB == 2), "tensor memory split");
     static constexpr int cols = 512 / kMinB;                              // of a CTA
     static constexpr int units = cols / (T / 128) / 4;                     // a thread can keep there
     __device__ static unsigned base(unsigned at) {

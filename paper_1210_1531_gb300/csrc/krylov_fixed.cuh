@@ -107,14 +107,10 @@ __device__ __forceinline__ void fx_tmem_st(unsigned at, const int4 v) {
 template <int N>
 __device__ __forceinline__ void fx_tmem_ld(unsigned at, int step, int4 (&v)[N]) {
     __syncwarp();
-    if constexpr (N == 1)
-        asm volatile(FX_LD(0, 1, 2, 3, 4) "tcgen05.wait::ld.sync.aligned;" : FX_OUT(v[0]) : "r"(at) : "memory");
-    else if constexpr (N == 2)
+    static_assert(N == 2 || N == 4, "units at a time");
+    if constexpr (N == 2)
         asm volatile(FX_LD(0, 1, 2, 3, 8) FX_LD(4, 5, 6, 7, 9) "tcgen05.wait::ld.sync.aligned;"
                      : FX_OUT(v[0]), FX_OUT(v[1]) : "r"(at), "r"(at + step) : "memory");
-    else if constexpr (N == 3)
-        asm volatile(FX_LD(0, 1, 2, 3, 12) FX_LD(4, 5, 6, 7, 13) FX_LD(8, 9, 10, 11, 14) "tcgen05.wait::ld.sync.aligned;"
-                     : FX_OUT(v[0]), FX_OUT(v[1]), FX_OUT(v[2]) : "r"(at), "r"(at + step), "r"(at + 2 * step) : "memory");
     else
         asm volatile(FX_LD(0, 1, 2, 3, 16) FX_LD(4, 5, 6, 7, 17) FX_LD(8, 9, 10, 11, 18) FX_LD(12, 13, 14, 15, 19)
                      "tcgen05.wait::ld.sync.aligned;"
