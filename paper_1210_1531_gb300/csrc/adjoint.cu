@@ -346,6 +346,8 @@ __device__ __forceinline__ void sampled_block(const AdjointArgs& g, const int* n
         const double* U = Uw[wi];
         const double* YH = YHw[wi];
         const double* YS = YSw[wi];
+        // (unrolled, this loop costs the kernel's other ones registers: 188.0 instead of 182.1 ms, 4096 atoms)
+#pragma unroll 1
         for (int n = 0; n < nvw[wi]; ++n) {
             double2 x0, x1, y0, y1, z0, z1;
             ld4(U + (size_t)n * vs + cp4, x0, x1);
