@@ -9,7 +9,9 @@
  * model of carbon.
  *
  * Conventions
- *   Units      eV, Angstrom. All floating point is IEEE double (FP64).
+ *   Units      eV, Angstrom. All floating point is IEEE double (FP64). Inside the Krylov build
+ *              of most systems vectors are 57-bit integers with one scale each (the first steps,
+ *              and the scalars of every step, in FP64); its errors are those of the FP64 build.
  *   Basis      N atoms, M = 4N orbitals; basis index j = 4*J + alpha, alpha = (s, px, py, pz).
  *   Positions  double[N][3], row-major; orthorhombic periodic box; minimum-image convention
  *              (the box must exceed 2*r_cut, and 2*r_cluster when r_cluster > 0).
@@ -100,14 +102,16 @@ typedef struct elses_params {
                                (ignored when k3_ctas_per_sm is set)                              */
     int    graph;           /* 1: elses_energy_force replays its step as a CUDA graph: the first
                                call with a new launch plan runs as usual, the next captures the
-                               device work (columns, the bisection's fixed launch sequence,
-                               density, scalars, forces at the device-resident mu), later calls
+                               device work (columns, the bisection, the density, scalars,
+                               forces at the device-resident mu), later calls
                                replay it with one host synchronisation; a rebuild that keeps the
                                plan and buffers keeps the graph. Results equal the eager path.   */
-    int    k3_lanes;        /* lanes per column of the Krylov kernel: 0 = automatic (a half-warp
-                               per column, two columns per warp, for the size classes whose
-                               clusters would leave the last slot of 32 atoms at most half full;
-                               forces from the density matrix and per-column spaces only),
+    int    k3_lanes;        /* lanes per column of the FP64 Krylov kernels, which take what the
+                               fixed-point one does not (clusters past 336 atoms, rows of more
+                               than 64 blocks or of very different size): 0 = automatic (a
+                               half-warp per column, two columns per warp, for the size classes
+                               whose clusters would leave the last slot of 32 atoms at most half
+                               full; forces from the density matrix and per-column spaces only),
                                32 = one warp per column always                                   */
     int    max_qr_sweeps;   /* cap on the implicit-shift QR sweeps of one projected eigenproblem
                                (0: 30 nu); a column that needs more sets ELSES_ERR_TIMEOUT       */

@@ -32,12 +32,13 @@
 // the one that is not to run returns at once.
 //
 // Against an 80-bit recursion (48 columns of 512-atom systems, G at three energies, geometric mean
-// of the relative errors; FP64 kernel first, both with the same eigensolver but for its chase):
-// displaced diamond 7.7e-15 / 8.9e-15 with two classical passes and 8.7e-15 / 8.3e-15 with the second
-// from S'; dense disordered carbon 1.11e-14 / 1.40e-14 and 1.19e-14 / 1.40e-14; the same H and S as a
-// caller's: 8.3e-15 / 8.0e-15, 7.9e-15 / 8.7e-15, 1.12e-14 / 1.30e-14, 1.04e-14 / 1.25e-14. Whole density
-// matrices of 512 atoms against dense 64-bit references, mean of eight: 4.7e-15 / 4.9e-15; G: 3.1e-13 /
-// 2.3e-13.
+// of the relative errors; FP64 kernel and the longer chase first): displaced diamond 7.7e-15 / 7.1e-15
+// with two classical passes and 8.7e-15 / 8.0e-15 with the second from S'; dense disordered carbon 1.11e-14 /
+// 1.18e-14 and 1.19e-14 / 1.17e-14; the same H and S as a caller's: 8.3e-15 / 7.2e-15, 7.9e-15 / 7.5e-15,
+// 1.12e-14 / 1.10e-14, 1.04e-14 / 1.31e-14. rho of 256 columns of graphite with grains: geometric mean
+// 7.0e-16 / 6.8e-16, largest 1.1e-14 / 3.7e-14 (one column). rho with one way of Gram-Schmidt against the other, all
+// columns, root mean square: graphite with grains 1.6e-15 / 0.8e-15, diamond (4096) 5.1e-16 / 2.9e-16,
+// disordered carbon (4096) 3.1e-15 / 4.7e-15; poles, median 4 to 11e-14 / 2 to 4e-14 eV.
 #include <algorithm>
 
 #include "krylov.cuh"
@@ -381,8 +382,8 @@ __device__ __forceinline__ int2 fx_hi(const int4& v) { return make_int2(v.z, v.w
 // differ most, FP64 kernel first: graphite with diamond grains (32768 atoms) 2.6e-10 / 2.6e-10, dense
 // disordered carbon (4096) 1.2e-10 / 1.0e-10, diamond (4096) 5.6e-11 / 5.7e-11. (With six steps whatever
 // the amplitudes, and their vectors subtracted as integers, the first was 1.2e-9 and rho there off by 6e-12.)
-// Each step costs 3% of the kernel. kLead 6 and kSmall 10, in ms: diamond 33.2 (32.9 with six steps
-// always), disordered carbon (65536) 303 (298), graphite with grains 184 (156): a third of its atoms have
+// Each step costs 3% of the kernel. kLead 6 and kSmall 10, in ms: diamond 33.3 (32.9 with six steps
+// always), disordered carbon (65536) 303 (299), graphite with grains 184 (154): a third of its atoms have
 // neighbours behind weak bonds. kSmall 12: 177 there, but poles off by 3.0e-10; kSmall 8: 193, 34.3 and 314.
 constexpr int kLead = 6, kSmall = 10;
 

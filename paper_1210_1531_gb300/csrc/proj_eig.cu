@@ -9,9 +9,9 @@
 // GB300 form. On this part the FP64 pipe charges a whole warp instruction whatever the number
 // of active lanes, so every FP64 instruction must carry work on all lanes:
 //   k_eig_reduce   one warp per column, matrices in shared memory: Cholesky (or, where S' = I to
-//                  2^-40, its first-order form), the reduction A = L^-1 H' L^-T and the Householder reduction of A to tridiagonal form T
-//                  (lanes over rows / columns); the three vectors z = L^-1 (U, SU, HU)_j are
-//                  reflected along, y = Q_H^T z.
+//                  2^-40, its first-order form), the reduction A = L^-1 H' L^-T and the Householder
+//                  reduction of A to tridiagonal form T (lanes over rows / columns); the three
+//                  vectors z = L^-1 (U, SU, HU)_j are reflected along, y = Q_H^T z.
 //   k_eig_chase    one thread per column: implicit-shift QR sweeps on T (Wilkinson shift, Givens
 //                  bulge chase) -- the sequential part; the rotations are recorded. A warp issues one
 //                  FP64 instruction in 64 clocks and there is less than one warp per scheduler up to
