@@ -7,7 +7,17 @@ import re
 SOURCE = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1210_1531_gb300", "csrc",
                       "krylov_fixed.cu")
 CLEAR = re.compile(r"st\.(bits|top)\[\d\]\[threadIdx\.x\] = [^;]*\b0;")
-GATHER = re.compile(r"\b(fx_update|fx_products|fx_products_lead|fx_products_dense)<")
+
+
+def source():
+    with open(SOURCE) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def gathering_phases(text):
+    """The device functions that end in the atomics."""
+    return {re.findall(r"__forceinline__ void (fx_\w+)\(", text[:m.start()])[-1]
+            for m in re.finditer(r"fx_(?:or|max)<NC>\(m", text)}
 
 
 def unconditional(text):
@@ -20,24 +30,16 @@ def unconditional(text):
 
 
 def test_a_barrier_follows_every_clearing():
-    with open(SOURCE) as f:
-        text = re.sub(r"//[^\n]*", "", f.read())
+    text = source()
+    phases = gathering_phases(text)
+    assert {"fx_update", "fx_products"} <= phases
+    gather = re.compile(r"\b(%s)<" % "|".join(sorted(phases, key=len, reverse=True)))
     kernel = text[text.index(") k_krylov_fixed("):]
     kernel = kernel[:kernel.index("\nnamespace {")]
+    assert phases == {m.group(1) for m in gather.finditer(kernel)}      # every one is called in the loop
     clears = [m.end() for m in CLEAR.finditer(kernel)]
     assert len(clears) >= 4
     for at in clears:
-        following = GATHER.search(kernel, at)
-        end = following.start() if following else len(kernel)
+        following = gather.search(kernel, at)
         if following:
-            assert "__syncthreads();" in unconditional(kernel[at:end]), kernel[at - 80:end + 20]
-
-
-def test_the_gathers_are_where_the_loop_calls_them():
-    """The phases the rule above looks for are the ones that end in the atomics."""
-    with open(SOURCE) as f:
-        text = f.read()
-    names = set()
-    for m in re.finditer(r"fx_(?:or|max)<NC>\(m", text):
-        names.add(re.findall(r"__forceinline__ void (fx_\w+)\(", text[:m.start()])[-1])
-    assert names == {"fx_products", "fx_products_dense", "fx_products_lead", "fx_update"}
+            assert "__syncthreads();" in unconditional(kernel[at:following.start()]), kernel[at - 80:following.end()]
