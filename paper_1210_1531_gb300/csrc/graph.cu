@@ -71,7 +71,7 @@ std::vector<long long> graph_key(elses_system s, const double* forces_dev) {
     add_bytes(&s->skd, sizeof(s->skd));
     for (int b = 0; b < s->n; b += s->batch_atoms) k.push_back(s->h_row_ptr[b]);   // batch pattern offsets
     for (const auto& L : s->k3_launches) {
-        k.insert(k.end(), {L.batch_begin, L.batch_end, L.item_begin, L.item_count, L.na, L.grid, L.bps, L.fx, L.fx_dense, L.grid64, L.bps64,
+        k.insert(k.end(), {L.batch_begin, L.batch_end, L.item_begin, L.item_count, L.na, L.grid, L.bps, L.fx, L.fx_dense, L.fx_b, L.grid64, L.bps64,
                            (long long)L.scratch_off});
     }
     return k;

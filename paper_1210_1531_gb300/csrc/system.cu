@@ -181,7 +181,7 @@ int prepare_columns(elses_system s) {
             }
             if (fx >= 0) bps = shape(true, fx_b, fx_b);
             const int grid = std::min(fx >= 0 ? fx_items(fx, count) : count, s->num_sms * bps);
-            s->k3_launches.push_back({b, e, begin, count, na, grid, bps, half ? 1 : 0, key, fx, fx_dense, grid64, bps64, batch_off});
+            s->k3_launches.push_back({b, e, begin, count, na, grid, bps, half ? 1 : 0, key, fx, fx_dense, fx_b, grid64, bps64, batch_off});
             // scratch for the kernel with the largest need, as caller matrices change it without a new plan
             const size_t fp64 = (size_t)grid64 * kWarpsPerAtom * 2 * nm * na * 4;
             const size_t fixed = fx >= 0 || fx_dense >= 0 ? (size_t)std::min(fx_items(form, count), s->num_sms * fx_b) * fx_scratch_doubles(form, nm, na) : 0;
@@ -469,7 +469,8 @@ static void launch_class(elses_system s, KrylovArgs ka, const elses_system_s::K3
     const int form = !s->user_hs ? L.fx : s->fx_user ? L.fx_dense : -1;
     ka.na_max = L.na;
     if (form >= 0) {
-        int bps = fx_blocks_per_sm(form, L.na, s->max_nb + 1, s->nu_max, s->p.reorth != 0, store);
+        // (no more CTAs than the plan has scratch for, also where the form without kept bases would fit more)
+        int bps = std::min(L.fx_b, fx_blocks_per_sm(form, L.na, s->max_nb + 1, s->nu_max, s->p.reorth != 0, store));
         if (!s->user_hs) bps = std::min(bps, L.bps);
         else if (s->p.k3_ctas_per_sm > 0) bps = std::min(bps, s->p.k3_ctas_per_sm);
         launch_krylov(s, ka, form, std::min(fx_items(form, ka.n_items), s->num_sms * bps), bps, st);

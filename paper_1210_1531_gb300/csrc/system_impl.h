@@ -117,9 +117,10 @@ struct elses_system_s {
     // batch can run at the same time
     // key: the class's bound on cluster size in slots of 16 atoms (its capacity na may be larger)
     // fx: the form of the fixed-point kernel that runs the class, -1 the FP64 kernels
-    // and fx_dense with caller matrices; grid64, bps64: the FP64 kernels' shape
+    // and fx_dense with caller matrices; fx_b: its CTAs per SM that the plan has scratch for; grid64,
+    // bps64: the FP64 kernels' shape
     struct K3Launch {
-        int batch_begin, batch_end, item_begin, item_count, na, grid, bps, half, key, fx, fx_dense, grid64, bps64;
+        int batch_begin, batch_end, item_begin, item_count, na, grid, bps, half, key, fx, fx_dense, fx_b, grid64, bps64;
         size_t scratch_off;
     };
     bool fx = false;                       // the fixed-point Krylov form suits the system's H and S

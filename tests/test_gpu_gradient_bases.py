@@ -70,11 +70,12 @@ def test_same_with_and_without_kept_bases(n, nu, r_cluster, reorth, caller):
         assert float((a + b - w).abs().max()) <= 4.0 * 2.0 ** -53 * float(torch.maximum(a.abs(), b.abs()).max())
 
 
-@pytest.mark.parametrize("n, nu, r_cluster", [(64, 30, 0.0), (512, 24, 4.4), (4096, 8, 4.0)])
-def test_two_pass(n, nu, r_cluster):
+@pytest.mark.parametrize("n, nu, r_cluster", [(64, 30, 0.0), (211, 20, 0.0), (512, 24, 4.4), (4096, 8, 4.0)])
+@pytest.mark.parametrize("caller", ["", "own"])
+def test_two_pass(n, nu, r_cluster, caller):
     """V formed by another kernel: the same to rounding, for spaces far from exhausted."""
-    kept = _system(n, nu, r_cluster, "", exact_forces=True, reorth=1)
-    two = _system(n, nu, r_cluster, "", exact_forces=True, reorth=1, two_pass=True)
+    kept = _system(n, nu, r_cluster, caller, exact_forces=True, reorth=1)
+    two = _system(n, nu, r_cluster, caller, exact_forces=True, reorth=1, two_pass=True)
     mu, _ = kept.find_mu()
     for w, g in zip(kept.omega_gradient(mu), two.omega_gradient(mu)):
         assert float((g - w).abs().max()) <= 1e-11 * float(w.abs().max())
